@@ -217,6 +217,98 @@ def run(s):
                 accepted=np.array(stats.accept_len[:]))
 
 
+# ------------------------------------------------------------------------------------ in 64 bits
+def _mat64(w, name, bits):
+    """A weight matrix in float64; with bits = 8 as the quantised target holds it (per row: scale =
+    max / 127, codes rounded half to even, scale and quotient in float32)."""
+    t = w[name]
+    if bits != 8:
+        return t.double()
+    f = t.float()
+    top = f.abs().amax(dim=1, keepdim=True)
+    scale = top / torch.full_like(top, 127.0)
+    scale[scale == 0] = 1.0
+    return (f / scale).round_().clamp_(-127, 127).double() * scale.double()
+
+
+def _decode64(m, w, x, pos, parts, bits):
+    """The decoder over the rows x at RoPE positions pos; parts = (first row, rows, mask) of every
+    episode. Returns the final-norm output."""
+    half, n = m.head_dim // 2, x.shape[0]
+    ang = pos.double()[:, None] * m.rope_theta ** (-torch.arange(half, device=x.device, dtype=torch.float64) / half)
+    cos, sin = ang.cos()[:, None], ang.sin()[:, None]
+
+    def norm(v, gain):
+        return v * torch.rsqrt((v * v).mean(dim=1, keepdim=True) + m.rms_eps) * w[gain].double()
+
+    def rotate(v):
+        a, b = v[..., :half], v[..., half:]
+        return torch.cat((a * cos - b * sin, b * cos + a * sin), dim=-1)
+
+    for i in range(m.n_layers):
+        p = "layers.%d." % i
+        q, k, v = (norm(x, p + "norm1") @ _mat64(w, p + "wqkv", bits).T).view(n, 3, m.n_heads, m.head_dim).unbind(1)
+        q, k = rotate(q), rotate(k)
+        out = torch.empty_like(v)
+        for r0, rows, mask in parts:
+            s = slice(r0, r0 + rows)
+            a = torch.einsum("thd,shd->hts", q[s], k[s]) * m.head_dim ** -0.5
+            a = a.masked_fill(~mask, -math.inf).softmax(dim=-1)
+            out[s] = torch.einsum("hts,shd->thd", a, v[s])
+        x = x + out.reshape(n, -1) @ _mat64(w, p + "wo", bits).T
+        gate, up = (norm(x, p + "norm2") @ _mat64(w, p + "wgu", bits).T).chunk(2, dim=1)
+        x = x + (torch.nn.functional.silu(gate) * up) @ _mat64(w, p + "wd", bits).T
+    return norm(x, "final_norm")
+
+
+def _inputs64(w, embeds, ids):
+    ids = torch.tensor(ids, device="cuda")
+    return torch.where((ids < 0)[:, None], embeds, w["embed"][ids.clamp(min=0)]).double()
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits. None for a chunk: its tokens are whole values."""
+    if case["kind"] == "chunk":
+        return None
+    rng = random.Random(seed)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    if case["kind"] == "gemm":
+        x = torch.randn(case["t"], case["k"], generator=g, device="cuda", dtype=torch.float32)
+        w = torch.randn(case["n"], case["k"], generator=g, device="cuda", dtype=torch.bfloat16).mul_(0.02)
+        return x.double() @ w.double().T
+    m, w, bits = MODELS[case["model"]], _weights(case["model"]), case["bits"]
+    act = slice(m.action_base, m.action_base + m.n_bins)
+    if case["kind"] == "score":
+        n, rows = case["prefix"], case["rows"]
+        embeds, ids = _prefix(m, [n], min(256, n // 2), g, rng)
+        tree = _tree(m, rows, rng)
+        mask = torch.ones(n + rows, n + rows, dtype=torch.bool, device="cuda").tril_()
+        mask[n:, n:] = False
+        sees = np.zeros((rows, rows), dtype=bool)
+        for i, p in enumerate(tree["parent"]):
+            if p >= 0:
+                sees[i] = sees[p]
+            sees[i, i] = True
+        mask[n:, n:] = torch.from_numpy(sees).cuda()
+        pos = torch.tensor(list(range(n)) + [n + d for d in tree["depth"]], device="cuda")
+        x = _inputs64(w, torch.cat((embeds, embeds.new_zeros(rows, m.d_model))), ids + tree["tokens"])
+        h = _decode64(m, w, x, pos, [(0, n + rows, mask)], bits)
+        top = (h[n:] @ _mat64(w, "lm_head", bits)[act].T).topk(2, dim=1)
+        return dict(greedy=(top.indices[:, 0] + m.action_base).cpu().numpy(),
+                    margin=(top.values[:, 0] - top.values[:, 1]).cpu())
+    lens = [case["visual"] + rng.randint(case["text_lo"], case["text_hi"]) for _ in range(case["episodes"])]
+    embeds, ids = _prefix(m, lens, case["visual"], g, rng)
+    parts, r0 = [], 0
+    for n in lens:
+        parts.append((r0, n, torch.ones(n, n, dtype=torch.bool, device="cuda").tril_()))
+        r0 += n
+    pos = torch.cat([torch.arange(n, device="cuda") for n in lens])
+    h = _decode64(m, w, _inputs64(w, embeds, ids), pos, parts, bits)
+    logits = h[[r + n - 1 for r, n, _ in parts]] @ _mat64(w, "lm_head", bits).T
+    return dict(first=(logits[:, act].argmax(dim=1) + m.action_base).cpu().numpy(), logits=logits)
+
+
 # ------------------------------------------------------------------------------------ work and tolerance
 def _forward(m, rows, keys, n_ep, heads, bits):
     """(bytes, flops) of one forward of the target over `rows` rows of n_ep episodes with `keys` visible
