@@ -30,6 +30,11 @@ namespace gemm_ck {
 using namespace gemm_tc;
 
 constexpr int MAX_S = 8;                   // largest cluster = K slices per tile (portable limit)
+// Row chunks whose CTAs run side by side: 12 chunks x 12 tiles (what 148 SMs run at once) read least
+// of both operands. In tile-first order every wave of a long launch streams the whole matrix again
+// (gate/up of 4764 rows: 22 times 180 MB); 16 prefixes of 296 rows: 132 -> 115 ms (980 W either way:
+// these launches run at the power limit, and bytes are power).
+constexpr int RASTER = 12;
 constexpr long FIXED_CLOCKS = 12000;       // start, accumulator read-out and exit of a CTA (cost estimate of a launch plan)
 
 __device__ __forceinline__ uint32_t cluster_size() {
@@ -100,7 +105,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   constexpr int ROPE_ROWS = ROPE_SMEM ? 32 : 1, ROPE_HALF = ROPE_SMEM ? 64 : 1;
   __shared__ __align__(16) float2 s_rope[ROPE_ROWS * ROPE_HALF];
   __shared__ float s_red[8][MAX_T];
-  __shared__ int s_flag[8];
+  __shared__ int s_flag;
   __shared__ float s_xv[4][2];             // EPI_TOPK: exchange between the two warps of a row group
   __shared__ int s_xi[4][2];
 
@@ -108,18 +113,27 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int S = (int)cluster_size();
   const int rank = (int)cluster_rank();
   constexpr bool swiglu = MODE == EPI_SWIGLU;
-  const int tile = blockIdx.x / S;
+  // Order in which clusters take (tile, row chunk) pairs: groups of ea.raster chunks, within a group
+  // tile after tile with its chunks side by side, so that what runs at the same time shares weights
+  // and rows in L2.
+  int tile = (int)blockIdx.x / S, chunk = (int)blockIdx.y;
+  if (TN == MAX_T && gridDim.y > 1) {
+    const int n_tiles = (int)gridDim.x / S, c = chunk * n_tiles + tile;
+    const int grp = c / (ea.raster * n_tiles), in = c - grp * ea.raster * n_tiles;
+    const int width = min(ea.raster, (int)gridDim.y - grp * ea.raster);
+    tile = in / width;
+    chunk = grp * ea.raster + in - tile * width;
+  }
   const int kb0 = rank * KB / S, kb1 = (rank + 1) * KB / S;
   const int n_units = kb1 - kb0;
   const long long u0 = (long long)tile * KB + kb0;
   const int tiles = gridDim.x / S;
-  // rows of this CTA: the blockIdx.y-th chunk. The 128-row instantiation takes its chunk length
+  // rows of this CTA: one chunk. The 128-row instantiation takes its chunk length
   // and MMA width from the launch (rows are spread evenly over the chunks of a long launch, so the
   // width is rarely the full 128); the last chunk has a tensor map with its own box.
-  const int row0 = ea.row0 + (int)blockIdx.y * ea.chunk_rows;
-  const int T = ea.T - (int)blockIdx.y * ea.chunk_rows < ea.chunk_rows ? ea.T - (int)blockIdx.y * ea.chunk_rows
-                                                                         : ea.chunk_rows;
-  const bool tail = blockIdx.y == gridDim.y - 1;
+  const int row0 = ea.row0 + chunk * ea.chunk_rows;
+  const int T = min(ea.T - chunk * ea.chunk_rows, ea.chunk_rows);
+  const bool tail = chunk == (int)gridDim.y - 1;
   const int tn = TN == MAX_T ? (tail ? ea.tn_tail : ea.tn_chunk) : TN;
   const CUtensorMap *xmap = (TN == MAX_T && tail) ? &tmXtail : &tmX;
   constexpr int W_LOAD_BYTES = Q8 ? W_STAGE_BYTES / 2 : W_STAGE_BYTES;   // int8 codes: half the bytes from HBM
@@ -336,11 +350,15 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
     bool have = n_units > 0;
     if (have) {
-      const bool mine = mbar_wait(tfull_bar, 0, ea.wait_ns);
-      if (lane == 0) s_flag[warp - 2] = mine ? 1 : 0;
+      // one thread polls and the others sleep at the barrier (256 polling threads cost power and
+      // shared-memory cycles for the whole stream)
+      if (et == 0) {
+        const bool done = mbar_wait(tfull_bar, 0, ea.wait_ns);
+        s_flag = done ? 1 : 0;
+        if (!done) atomicExch(err, SV_ERR_WAIT_TMEM_FULL);
+      }
       epi_barrier();
-      have = s_flag[0] && s_flag[1] && s_flag[2] && s_flag[3] && s_flag[4] && s_flag[5] && s_flag[6] && s_flag[7];
-      if (!have && et == 0) atomicExch(err, SV_ERR_WAIT_TMEM_FULL);
+      have = s_flag != 0;
       tc_fence_after();
       if (rope_ring) {
         const int hp = ea.dh >> 2;                         // 16-byte pieces (two pairs) per row

@@ -390,6 +390,7 @@ int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs
   ea.row0 = 0;
   ea.T = R;
   ea.chunk_rows = plan.chunk_rows;
+  ea.raster = gemm_ck::RASTER;
   ea.tn_chunk = plan.tn_chunk;
   ea.tn_tail = plan.tn_tail;
   ea.pf_w = nullptr;
@@ -1855,6 +1856,7 @@ static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, i
   ea.row0 = 0;
   ea.T = T;
   ea.chunk_rows = plan.chunk_rows;
+  ea.raster = gemm_ck::RASTER;
   ea.tn_chunk = plan.tn_chunk;
   ea.tn_tail = plan.tn_tail;
   if (!gemm_tc::make_x_map(&mx[0], limbs, nx, T, K, plan.tn_chunk) ||

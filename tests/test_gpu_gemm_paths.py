@@ -1,0 +1,26 @@
+"""The stand-alone product at the sizes where its launch plans change, against float64."""
+import pytest
+import torch
+
+from synth_inputs import rng
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(T, N, K, packed):
+    from paper_2507_22424_b200.binding import gemm, gemm_prepacked, pack_weights
+    x = rng.normal(21, 1, (T, K), 1.0, dtype=torch.float32)
+    w = rng.normal_bf16(21, 2, (N, K), 0.02)
+    ref = x.double() @ w.double().T
+    y = (gemm_prepacked(x.cuda(), pack_weights(w.cuda()), N) if packed else gemm(x.cuda(), w.cuda())).cpu().double()
+    # two-limb activations (2^-18 relative) and fp32 accumulation; outputs ~0.02 * sqrt(K)
+    tol = 1e-4 * 0.02 * (K ** 0.5) + 1e-6
+    assert (y - ref).abs().max() < tol, float((y - ref).abs().max())
+
+
+# more row chunks than run side by side: a full group and a last one of one or several chunks, a ragged
+# last chunk, one tile and several, with and without K slices
+@pytest.mark.parametrize("T,N,K", [(1537, 512, 64), (1665, 1000, 256), (3100, 256, 1024), (2049, 768, 520)])
+@pytest.mark.parametrize("packed", [True, False])
+def test_many_row_chunks(T, N, K, packed):
+    _check(T, N, K, packed)
