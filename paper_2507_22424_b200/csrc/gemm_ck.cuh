@@ -109,7 +109,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __shared__ float s_xv[4][2];             // EPI_TOPK: exchange between the two warps of a row group
   __shared__ int s_xi[4][2];
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const int S = (int)cluster_size();
   const int rank = (int)cluster_rank();
   constexpr bool swiglu = MODE == EPI_SWIGLU;
@@ -141,7 +141,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint32_t idesc = instr_desc(2 * tn);
 
   const int npre = n_units < STAGES ? n_units : STAGES;
-  uint64_t pol_w = 0;
+  const uint64_t pol_w = policy_evict_first();
   // test hook: the K block that is never loaded (-1: none)
   const int withheld = ea.withhold_unit - 1;
   auto load_w = [&](int it) {
@@ -178,7 +178,6 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     grid_dep_launch();
-    pol_w = policy_evict_first();
     for (int it = 0; it < npre; it++) load_w(it);
   }
   if (warp == 1) {
@@ -190,6 +189,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   tc_fence_after();
   uint32_t tmem_base;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
+  tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0);
 
   // finishing-loop operands that the epilogue warps fetch while the MMAs run (part 1)
   const bool rope_staged = MODE == EPI_QKV && T <= ROPE_ROWS && (ea.dh >> 1) <= ROPE_HALF;
@@ -203,48 +203,66 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0 && n_units > 0) {
-      const uint64_t pol_x = policy_evict_last();
-      grid_dep_wait();
-      for (int j = 0; j < npre; j++)
-        if (j != withheld)
-          tma_load_3d(base + RING0 + j * STAGE + XOFF, xmap, (kb0 + j) * BK, row0, 0, full_bar(j), pol_x);
-      for (int it = npre; it < n_units; it++) {
-        const int st = it % STAGES, rnd = it / STAGES;
-        if (!mbar_wait(empty_bar(st), (rnd - 1) & 1, ea.wait_ns)) {
-          atomicExch(err, SV_ERR_WAIT_EMPTY);
-          break;
-        }
+    const uint64_t pol_x = policy_evict_last();
+    const bool lead = elect_one();
+    grid_dep_wait();
+    auto load_x = [&](int it, int st) {
+      if (it != withheld)
+        tma_load_3d(base + RING0 + st * STAGE + XOFF, xmap, (kb0 + it) * BK, row0, 0, full_bar(st), pol_x);
+    };
+    if (lead)
+      for (int j = 0; j < npre; j++) load_x(j, j);
+    __syncwarp();
+    for (int it = npre, st = 0, ph = 0; it < n_units; it++) {
+      const bool ok = mbar_wait(empty_bar(st), ph, ea.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lead) atomicExch(err, SV_ERR_WAIT_EMPTY);
+        break;
+      }
+      if (lead) {
         load_w(it);
-        if (it != withheld)
-          tma_load_3d(base + RING0 + st * STAGE + XOFF, xmap, (kb0 + it) * BK, row0, 0, full_bar(st), pol_x);
+        load_x(it, st);
+      }
+      __syncwarp();
+      if (++st == STAGES) {
+        st = 0;
+        ph ^= 1;
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && n_units > 0) {
-      for (int it = 0; it < n_units; it++) {
-        const int st = it % STAGES, rnd = it / STAGES;
-        if (!mbar_wait(Q8 ? conv_bar(it % NE) : full_bar(st), Q8 ? (it / NE) & 1 : rnd & 1, ea.wait_ns)) {
-          atomicExch(err, SV_ERR_WAIT_FULL);
-          break;
-        }
-        tc_fence_after();
-        const uint32_t sW = Q8 ? base + (it % NE) * W_STAGE_BYTES : base + st * STAGE;
-        const uint32_t sX = base + RING0 + st * STAGE + XOFF;
+    const bool lead = elect_one();
+    for (int it = 0, st = 0, ph = 0, e = 0, eph = 0; it < n_units; it++) {
+      const bool ok = mbar_wait(Q8 ? conv_bar(e) : full_bar(st), Q8 ? eph : ph, ea.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lead) atomicExch(err, SV_ERR_WAIT_FULL);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t sW = Q8 ? base + e * W_STAGE_BYTES : base + st * STAGE;
+      const uint32_t sX = base + RING0 + st * STAGE + XOFF;
+      const uint64_t adesc = smem_desc(sW), bdesc = smem_desc(sX);
+      if (lead) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; kk++) {
+        for (int kk = 0; kk < BK / 16; kk++)
 #pragma unroll
-          for (int h = 0; h < 2; h++) {
-            const uint64_t adesc = smem_desc(sW + h * (128 * BK * 2) + kk * 32);
-            const uint32_t d = tmem_base + (uint32_t)(h * AW);
-            tc_mma(d, adesc, smem_desc(sX + kk * 32), idesc, (it == 0 && kk == 0) ? 0u : 1u);
-          }
-        }
+          for (int h = 0; h < 2; h++)
+            // (descriptor addresses count 16 bytes)
+            tc_mma(tmem_base + (uint32_t)(h * AW), adesc + (uint64_t)((h * (128 * BK * 2) + kk * 32) >> 4),
+                   bdesc + (uint64_t)(kk * 2), idesc, (it == 0 && kk == 0) ? 0u : 1u);
         tc_commit(empty_bar(st));
-        if (Q8) tc_commit(efree_bar(it % NE));
+        if (Q8) tc_commit(efree_bar(e));
         if (it == n_units - 1) tc_commit(tfull_bar);
+      }
+      __syncwarp();
+      if (++st == STAGES) {
+        st = 0;
+        ph ^= 1;
+      }
+      if (++e == NE) {
+        e = 0;
+        eph ^= 1;
       }
     }
     __syncwarp();

@@ -150,6 +150,22 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+// One lane of a converged warp. The loops that issue MMAs and copies are run by all lanes of their
+// warp, with a vote where a lane could leave alone, and only the instructions themselves by the
+// elected lane: these instructions take their operands from uniform registers, and operands
+// computed under a one-lane branch have to be moved there one by one. With one-lane loops a K block
+// (eight MMAs, two waits, two commits) took the issuing thread about 0.5 us whatever its size, which
+// bounded every launch whose CTAs have 64 of them: a verification step of 27 rows took 3.20 ms
+// instead of 3.00, of one row 3.03 instead of 2.81.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
 // 16 consecutive fp32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
