@@ -51,52 +51,85 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__host__ __device__ constexpr int ck_tmem_cols(int TN) { return 2 * acc_width(TN) < 32 ? 32 : 2 * acc_width(TN); }
-
-// Quantised weights (Q8): a stage holds the int8 codes of a unit (16 KB from HBM) and its X slice;
-// the bf16 image the tensor cores read is written by the epilogue warps into one of two 32 KB
-// buffers in front of the ring. With half the bytes per unit the ring needs twice the units in
-// flight for the same HBM rate, so it takes all the shared memory there is.
-__host__ __device__ constexpr int q8_stage_bytes(int TN) { return W_STAGE_BYTES / 2 + 2 * TN * BK * 2; }
-// expanded buffers: as many units as can be in expansion at once (the expansion of a unit is a
-// chain of shared-memory latencies, barriers and a proxy fence of about a microsecond)
-__host__ __device__ constexpr int q8_expanded(int TN) { return TN <= 32 ? 3 : 2; }
-__host__ __device__ constexpr int q8_stages(int TN) {
-  return (216 * 1024 - q8_expanded(TN) * W_STAGE_BYTES) / q8_stage_bytes(TN) > 8
-             ? 8
-             : (216 * 1024 - q8_expanded(TN) * W_STAGE_BYTES) / q8_stage_bytes(TN);
-}
+// Quantised weights (Q8). The epilogue warps expand the int8 codes of a unit to bf16 straight into
+// tensor memory, where the MMAs read them as their A operand: a thread owns a weight row (64 codes
+// in from shared memory, 32 columns of bf16 pairs out). Shared memory then carries per unit only
+// the codes (written once, read once) and X: 56 KB at 32 rows, against 152 KB for an image expanded
+// in shared memory, whose three 32 KB buffers, block barriers and proxy fences bounded the kernel: a verification step
+// of 27 rows takes 3.23 ms instead of 4.26, of 8 rows 3.03 instead of 4.03, of 100 rows 5.71 instead
+// of 6.07. What is left over the bf16 weights' 3.00 ms is the chain of a unit: codes landed, 0.4 us
+// of expansion, MMAs, commit.
+// TMEM: two accumulators of 2 TN columns, then q8_expanded(TN) buffers of 64 columns (two halves of
+// 128 rows x 64 K); 128 rows would leave no room for any, so Q8 chunks are at most 96 rows.
+// The codes have a ring of their own, free as soon as they are in registers; the X slot of a unit
+// goes with its expanded buffer (same index, freed by the same commit) and has a producer warp.
+constexpr int Q8_MAX_T = 96;
+constexpr int Q8_CODE_BYTES = W_STAGE_BYTES / 2;
+constexpr int Q8_STAGES = 8;
+__host__ __device__ constexpr int q8_rows(int TN) { return TN > Q8_MAX_T ? Q8_MAX_T : TN; }
+__host__ __device__ constexpr int q8_expanded(int TN) { return TN > 64 ? 2 : 4; }
+__host__ __device__ constexpr int q8_x_bytes(int TN) { return 2 * q8_rows(TN) * BK * 2; }
 __host__ __device__ constexpr int q8_smem_bytes(int TN) {
-  return q8_expanded(TN) * W_STAGE_BYTES + q8_stages(TN) * q8_stage_bytes(TN) + 1024 + 256;
+  return Q8_STAGES * Q8_CODE_BYTES + q8_expanded(TN) * q8_x_bytes(TN) + 1024 + 256;
 }
-// Expansion groups: one per expanded buffer (group g always writes buffer g and takes the units
-// g, g + NE, ...: it waits for the MMAs of its previous unit before anything else, which also tells
-// it that every earlier load has landed, so a mbarrier parity can never be read a phase late).
-__host__ __device__ constexpr int q8_group_threads(int TN) { return q8_expanded(TN) == 3 ? 64 : 128; }
+__host__ __device__ constexpr int ck_threads(bool Q8) { return Q8 ? THREADS + 32 : THREADS; }
+__host__ __device__ constexpr int ck_acc_width(int TN, bool Q8) { return Q8 ? 2 * q8_rows(TN) : acc_width(TN); }
+__host__ __device__ constexpr int ck_tmem_cols(int TN, bool Q8) {
+  return Q8 ? 512 : (2 * acc_width(TN) < 32 ? 32 : 2 * acc_width(TN));
+}
+// D[tmem] (+)= A[tmem] * B[smem]^T: A as bf16 pairs, lane = row, column = two consecutive K.
+__device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// 32 consecutive columns of this thread's TMEM lane.
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
+      ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]),
+        "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// Two int8 codes in bytes 0 and 2 of w -> their bf16 images, exact: 128 + (low seven bits) and 128 or
+// 256 (by the sign bit) are bf16 values that one mask and one OR build; their difference is the code.
+__device__ __forceinline__ uint32_t codes_to_bf16x2(uint32_t w) {
+  const uint32_t a = (w & 0x007f007fu) | 0x43004300u, b = (w & 0x00800080u) | 0x43004300u;
+  const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162 *>(&a), *reinterpret_cast<const __nv_bfloat162 *>(&b));
+  return *reinterpret_cast<const uint32_t *>(&r);
+}
 
 // EpiArgs as in gemm_tc: the mode is a template parameter. KB = K blocks per tile.
 template <int TN, int MODE, bool Q8>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(ck_threads(Q8), 1)
 gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                const __grid_constant__ CUtensorMap tmXtail, const EpiArgs ea, const int KB,
                int *__restrict__ err) {
-  constexpr int STAGES = Q8 ? q8_stages(TN) : stages_of(TN);
-  constexpr int STAGE = Q8 ? q8_stage_bytes(TN) : stage_bytes(TN);
-  constexpr int NE = Q8 ? q8_expanded(TN) : 1;
-  constexpr uint32_t RING0 = Q8 ? NE * W_STAGE_BYTES : 0;     // Q8: the expanded weight buffers come first
-  constexpr uint32_t XOFF = Q8 ? W_STAGE_BYTES / 2 : W_STAGE_BYTES;   // X slice within a stage
-  constexpr int AW = acc_width(TN);
+  constexpr int STAGES = Q8 ? Q8_STAGES : stages_of(TN);
+  constexpr int STAGE = Q8 ? Q8_CODE_BYTES : stage_bytes(TN);
+  constexpr int NE = Q8 ? q8_expanded(TN) : 1;                // expanded buffers in TMEM
+  constexpr int RING_BYTES = STAGES * STAGE + (Q8 ? NE * q8_x_bytes(TN) : 0);
+  constexpr int AW = ck_acc_width(TN, Q8);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t bars = base + RING0 + STAGES * STAGE;
+  const uint32_t bars = base + RING_BYTES;
   auto full_bar = [&](int s) { return bars + 8u * s; };
   auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
   const uint32_t tfull_bar = bars + 8u * (2 * STAGES);
   const uint32_t tmem_slot = bars + 8u * (2 * STAGES + 1);
-  // Q8: expanded buffer e holds the bf16 image of a unit (conv) / has been read by its MMAs (efree)
+  // Q8: expanded buffer e holds the bf16 image of a unit (conv) / has been read by its MMAs, like X slot e (efree);
+  // X slot e, behind the codes, holds the unit's X (xfull)
   auto conv_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + e); };
   auto efree_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + NE + e); };
-  __shared__ int s_gflag[4];
+  auto xfull_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + 2 * NE + e); };
+  auto x_slot = [&](int e) { return base + (uint32_t)(STAGES * STAGE + e * q8_x_bytes(TN)); };
   __shared__ float s_scale[MAX_T];
   __shared__ int s_pos[MAX_T], s_slot[MAX_T], s_ep[MAX_T];
   // RoPE factors of the CTA's rows (EPI_QKV, up to 32 rows of up to 64 pairs): fetched while the
@@ -136,8 +169,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const bool tail = chunk == (int)gridDim.y - 1;
   const int tn = TN == MAX_T ? (tail ? ea.tn_tail : ea.tn_chunk) : TN;
   const CUtensorMap *xmap = (TN == MAX_T && tail) ? &tmXtail : &tmX;
-  constexpr int W_LOAD_BYTES = Q8 ? W_STAGE_BYTES / 2 : W_STAGE_BYTES;   // int8 codes: half the bytes from HBM
-  const uint32_t stage_tx = (uint32_t)(W_LOAD_BYTES + 2 * tn * BK * 2);
+  const uint32_t x_tx = (uint32_t)(2 * tn * BK * 2);
+  const uint32_t stage_tx = Q8 ? (uint32_t)Q8_CODE_BYTES : W_STAGE_BYTES + x_tx;
   const uint32_t idesc = instr_desc(2 * tn);
 
   const int npre = n_units < STAGES ? n_units : STAGES;
@@ -147,11 +180,11 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   auto load_w = [&](int it) {
     if (it == withheld) return;
     const int st = it % STAGES;
-    const uint32_t sW = base + RING0 + st * STAGE;
+    const uint32_t sW = base + st * STAGE;
     mbar_expect_tx(full_bar(st), stage_tx);
     if (Q8) {
       // the codes of the 256 x 64 tile; the epilogue warps expand them (below)
-      bulk_load(sW, ea.wq8 + (size_t)(u0 + it) * (BM * BK), W_STAGE_BYTES / 2, full_bar(st), pol_w);
+      bulk_load(sW, ea.wq8 + (size_t)(u0 + it) * (BM * BK), Q8_CODE_BYTES, full_bar(st), pol_w);
     } else if (ea.wpacked) {
       bulk_load(sW, ea.wpacked + (size_t)(u0 + it) * (BM * BK), W_STAGE_BYTES, full_bar(st), pol_w);
     } else {
@@ -167,13 +200,15 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     if (!ea.wpacked) prefetch_tensormap(&tmW);
     for (int s = 0; s < STAGES; s++) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), Q8 ? 2 : 1);     // Q8: the codes have been expanded AND the MMAs have read X
+      mbar_init(empty_bar(s), Q8 ? 4 : 1);     // Q8: one arrival per warp of the set that reads the codes
     }
-    if (Q8)
+    if (Q8) {
       for (int e = 0; e < NE; e++) {
-        mbar_init(conv_bar(e), 1);
+        mbar_init(conv_bar(e), 4);             // one arrival per warp of a set
         mbar_init(efree_bar(e), 1);
+        mbar_init(xfull_bar(e), 1);
       }
+    }
     mbar_init(tfull_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -181,7 +216,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     for (int it = 0; it < npre; it++) load_w(it);
   }
   if (warp == 1) {
-    tc_alloc(tmem_slot, ck_tmem_cols(TN));
+    tc_alloc(tmem_slot, ck_tmem_cols(TN, Q8));
     tc_relinquish();
   }
   tc_fence_before();
@@ -205,12 +240,12 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // ------------------------------------------------------------------ TMA producer
     const uint64_t pol_x = policy_evict_last();
     const bool lead = elect_one();
-    grid_dep_wait();
+    if (!Q8) grid_dep_wait();
     auto load_x = [&](int it, int st) {
       if (it != withheld)
-        tma_load_3d(base + RING0 + st * STAGE + XOFF, xmap, (kb0 + it) * BK, row0, 0, full_bar(st), pol_x);
+        tma_load_3d(base + st * STAGE + W_STAGE_BYTES, xmap, (kb0 + it) * BK, row0, 0, full_bar(st), pol_x);
     };
-    if (lead)
+    if (lead && !Q8)
       for (int j = 0; j < npre; j++) load_x(j, j);
     __syncwarp();
     for (int it = npre, st = 0, ph = 0; it < n_units; it++) {
@@ -221,7 +256,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
       if (lead) {
         load_w(it);
-        load_x(it, st);
+        if (!Q8) load_x(it, st);
       }
       __syncwarp();
       if (++st == STAGES) {
@@ -230,29 +265,55 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     }
     __syncwarp();
+  } else if (Q8 && warp == 10) {
+    // ------------------------------------------------------------------ X producer (Q8)
+    const uint64_t pol_x = policy_evict_last();
+    const bool lead = elect_one();
+    grid_dep_wait();
+    for (int it = 0, e = 0, ph = 1; it < n_units; it++) {
+      const bool ok = it < NE || mbar_wait(efree_bar(e), ph, ea.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lead) atomicExch(err, SV_ERR_WAIT_EMPTY);
+        break;
+      }
+      if (lead) {
+        mbar_expect_tx(xfull_bar(e), x_tx);
+        tma_load_3d(x_slot(e), xmap, (kb0 + it) * BK, row0, 0, xfull_bar(e), pol_x);
+      }
+      __syncwarp();
+      if (++e == NE) {
+        e = 0;
+        ph ^= 1;
+      }
+    }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     const bool lead = elect_one();
     for (int it = 0, st = 0, ph = 0, e = 0, eph = 0; it < n_units; it++) {
-      const bool ok = mbar_wait(Q8 ? conv_bar(e) : full_bar(st), Q8 ? eph : ph, ea.wait_ns);
+      const bool ok = Q8 ? mbar_wait(xfull_bar(e), eph, ea.wait_ns) && mbar_wait(conv_bar(e), eph, ea.wait_ns)
+                         : mbar_wait(full_bar(st), ph, ea.wait_ns);
       if (!__all_sync(0xffffffffu, ok)) {
         if (lead) atomicExch(err, SV_ERR_WAIT_FULL);
         break;
       }
       tc_fence_after();
-      const uint32_t sW = Q8 ? base + e * W_STAGE_BYTES : base + st * STAGE;
-      const uint32_t sX = base + RING0 + st * STAGE + XOFF;
+      const uint32_t sW = base + st * STAGE;
+      const uint32_t sX = Q8 ? x_slot(e) : sW + W_STAGE_BYTES;
+      const uint32_t tA = tmem_base + (uint32_t)(2 * AW + e * 64);         // Q8: the expanded weights
       const uint64_t adesc = smem_desc(sW), bdesc = smem_desc(sX);
       if (lead) {
 #pragma unroll
         for (int kk = 0; kk < BK / 16; kk++)
 #pragma unroll
-          for (int h = 0; h < 2; h++)
-            // (descriptor addresses count 16 bytes)
-            tc_mma(tmem_base + (uint32_t)(h * AW), adesc + (uint64_t)((h * (128 * BK * 2) + kk * 32) >> 4),
-                   bdesc + (uint64_t)(kk * 2), idesc, (it == 0 && kk == 0) ? 0u : 1u);
-        tc_commit(empty_bar(st));
-        if (Q8) tc_commit(efree_bar(e));
+          for (int h = 0; h < 2; h++) {
+            const uint32_t d = tmem_base + (uint32_t)(h * AW), acc = (it == 0 && kk == 0) ? 0u : 1u;
+            if (Q8)
+              tc_mma_ta(d, tA + (uint32_t)(h * 32 + kk * 8), bdesc + (uint64_t)(kk * 2), idesc, acc);
+            else                                   // (descriptor addresses count 16 bytes)
+              tc_mma(d, adesc + (uint64_t)((h * (128 * BK * 2) + kk * 32) >> 4), bdesc + (uint64_t)(kk * 2), idesc, acc);
+          }
+        tc_commit(Q8 ? efree_bar(e) : empty_bar(st));
         if (it == n_units - 1) tc_commit(tfull_bar);
       }
       __syncwarp();
@@ -304,67 +365,51 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     }
     if (Q8) {
-      // int8 -> bf16 expansion of every unit as it lands. NE groups of warps take the units in
-      // turn (group g: units g, g + NE, ... into expanded buffer g), so that NE units are in
-      // expansion at once; a thread owns every GT-th 16-byte piece of the codes (16 codes in, two
-      // 16-byte chunks of a 128-byte swizzled row out).
-      constexpr int GT = q8_group_threads(TN);
-      const int g = et / GT, gt = et - g * GT;
-      auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(2 + g), "n"(GT) : "memory"); };
-      if (g < NE) {
-        for (int it = g; it < n_units; it += NE) {
-          const int st = it % STAGES, rnd = it / STAGES, use = it / NE;
-          if (gt == 0) {
-            bool ok = true;
-            if (use > 0) ok = mbar_wait(efree_bar(g), (use - 1) & 1, ea.wait_ns);   // first: see above
-            if (ok) ok = mbar_wait(full_bar(st), rnd & 1, ea.wait_ns);
-            s_gflag[g] = ok ? 1 : 0;
-          }
-          group_sync();                                    // the buffer is free, the codes are there
-          if (!s_gflag[g]) {
-            if (gt == 0) atomicExch(err, SV_ERR_WAIT_FULL);
-            break;
-          }
-          const uint32_t sC = base + RING0 + st * STAGE, sE = base + g * W_STAGE_BYTES;
-          // A thread takes 16-byte pieces gt, gt + GT, ... of the unit's codes (piece p = codes
-          // 16 (p % 4) .. + 15 of row p / 4): consecutive lanes read consecutive shared memory, and
-          // the two 16-byte chunks each piece expands to land in their swizzled places.
-#pragma unroll 4
-          for (int p = gt; p < BM * 4; p += GT) {
-            const int r = p >> 2, q = p & 3;
-            uint32_t c[4];
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3]) : "r"(sC + p * 16) : "memory");
+      // int8 -> bf16 expansion of every unit as it lands. The four warps of a set (wp) take every second
+      // unit, a warp the lanes of quarter q of both halves: two units are in expansion at once. The
+      // codes of the set's next unit are read while the stores of this one drain.
+      const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * AW);
+      const uint32_t crow = base + (uint32_t)((q * 32 + lane) * 16);
+      uint32_t c[32];
+      auto fetch_codes = [&](int it) {
+        const int st = it % STAGES, rnd = it / STAGES;
+        if (!mbar_wait(full_bar(st), rnd & 1, ea.wait_ns)) return false;
 #pragma unroll
-            for (int h2 = 0; h2 < 2; h2++) {
-              // eight codes (two words) -> eight bf16, exact (|code| <= 127), on the integer and FMA
-              // pipes only: code + 128 in the low mantissa byte of 2^23, minus (2^23 + 128), gives the
-              // code as fp32, whose upper half is its bf16 image
-              const int ch = 2 * q + h2;
-              uint32_t o[4];
+        for (int k = 0; k < 8; k++)
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(c[4 * k]), "=r"(c[4 * k + 1]), "=r"(c[4 * k + 2]), "=r"(c[4 * k + 3])
+                       : "r"(crow + (uint32_t)(st * STAGE + (k & 3) * (BM * 16) + (k >> 2) * (128 * 16))) : "memory");
+        return true;
+      };
+      bool ok = wp >= n_units || fetch_codes(wp);
+      ok = __all_sync(0xffffffffu, ok);
+      for (int it = wp; ok && it < n_units; it += 2) {
+        if (lane == 0) mbar_arrive(empty_bar(it % STAGES));      // every lane has read its codes
+        const int e = it % NE, use = it / NE;
+        if (use > 0) ok = mbar_wait(efree_bar(e), (use - 1) & 1, ea.wait_ns);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
 #pragma unroll
-              for (int h = 0; h < 2; h++) {
-                const uint32_t x = c[2 * h2 + h] ^ 0x80808080u;
-                const float f0 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7650)) - 8388736.f;
-                const float f1 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7651)) - 8388736.f;
-                const float f2 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7652)) - 8388736.f;
-                const float f3 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7653)) - 8388736.f;
-                o[2 * h] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-                o[2 * h + 1] = __byte_perm(__float_as_uint(f2), __float_as_uint(f3), 0x7632);
-              }
-              asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(sE + r * 128 + ((ch ^ (r & 7)) << 4)),
-                           "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-            }
+        for (int h = 0; h < 2; h++) {
+          uint32_t o[32];
+#pragma unroll
+          for (int k = 0; k < 16; k++) {
+            o[2 * k] = codes_to_bf16x2(c[16 * h + k]);
+            o[2 * k + 1] = codes_to_bf16x2(c[16 * h + k] >> 8);
           }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
-          group_sync();                                    // the whole tile is written
-          if (gt == 0) {
-            mbar_arrive(conv_bar(g));
-            mbar_arrive(empty_bar(st));                    // the codes are no longer needed
-          }
+          tc_st32(trow + (uint32_t)(e * 64 + h * 32), o);
         }
+        const bool got = it + 2 < n_units ? fetch_codes(it + 2) : true;
+        tc_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(conv_bar(e));
+        ok = __all_sync(0xffffffffu, got);
       }
-      epi_barrier();                                       // the groups (and the idle warps) meet again
+      if (!ok && lane == 0) atomicExch(err, SV_ERR_WAIT_FULL);
+      __syncwarp();
+      epi_barrier();
     }
     bool have = n_units > 0;
     if (have) {
@@ -436,7 +481,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   }
 
-  if (warp >= 2) {
+  if (warp >= 2 && warp < 10) {
     // ------------------------------------------------------------------ epilogue, part 2:
     // rows rank, rank + S, ... of the tile. A thread owns four consecutive columns and every
     // RG-th of those rows (64 column groups x 4 row groups; SwiGLU, whose 128 outputs come
@@ -667,7 +712,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // before leaving (nobody leaves while a peer may still be reading its shared memory), so that
   // the barrier's latency passes behind the rest of the epilogue.
   if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  if (warp >= 2 && MODE == EPI_RESID) {
+  if (warp >= 2 && warp < 10 && MODE == EPI_RESID) {
     const int et = threadIdx.x - 64;
     epi_barrier();
     // thread i finishes this CTA's i-th row, which row group i % 4 (two warps) handled
@@ -686,7 +731,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1) tc_dealloc(tmem_base, ck_tmem_cols(TN));
+  if (warp == 1) tc_dealloc(tmem_base, ck_tmem_cols(TN, Q8));
 }
 
 template <int TN, int MODE, bool Q8>
@@ -698,7 +743,7 @@ inline cudaError_t launch_tq(const CUtensorMap &tmW, const CUtensorMap &tmX, con
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles * S, (ea.T + ea.chunk_rows - 1) / ea.chunk_rows);
-  cfg.blockDim = dim3(THREADS);
+  cfg.blockDim = dim3(ck_threads(Q8));
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
@@ -801,19 +846,21 @@ struct RowPlan {
   int chunks, chunk_rows, tn_chunk, tn_tail, S;
 };
 inline int ceil8(int x) { return (x + 7) / 8 * 8; }
-inline RowPlan plan_rows(int R, int tiles, int KB, const ClusterFit &fit) {
+// (q8: int8 weights, chunks of at most Q8_MAX_T rows)
+inline RowPlan plan_rows(int R, int tiles, int KB, const ClusterFit &fit, bool q8) {
+  const int max_rows = q8 ? Q8_MAX_T : MAX_T;
   RowPlan p = {1, MAX_T, tn_of(R), tn_of(R), 1};
-  if (R <= MAX_T) {
+  if (R <= max_rows) {
     if (R > 64) p.tn_chunk = p.tn_tail = ceil8(R);
     p.S = slices_for(tiles, KB, fit);
     return p;
   }
   const int fit1 = fit.max_active[1] > 0 ? fit.max_active[1] : 148;
-  const int cmin = (R + MAX_T - 1) / MAX_T;
+  const int cmin = (R + max_rows - 1) / max_rows;
   long best = -1;
   for (int c = cmin; c <= cmin + 6 && c <= R; c++) {
     const int rows = ceil8((R + c - 1) / c);               // chunk starts stay multiples of 8 rows
-    if (rows > MAX_T || (long)rows * (c - 1) >= R) continue;
+    if (rows > max_rows || (long)rows * (c - 1) >= R) continue;
     for (int S = 1; S <= MAX_S; S++) {
       const int fits = S == 1 ? fit1 : fit.max_active[S];
       if (fits <= 0 || (S > 1 && KB / S < 4)) continue;

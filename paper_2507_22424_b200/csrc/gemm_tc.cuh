@@ -220,8 +220,8 @@ struct EpiArgs {
   unsigned long long wait_ns;   // limit of every mbarrier wait
   int withhold_unit;     // test hook (specvla_gemm_fault_test): > 0: the producer of every CTA skips its
                          // (withhold_unit - 1)-th K block, so the waits for it run out; 0: off
-  const signed char *wq8;   // int8 codes of the weights in the same unit order (16 KB per unit, rows of 64
-                            // codes, not swizzled), or NULL; wscale[n] = scale of weight row n
+  const signed char *wq8;   // int8 codes of the weights in the same unit order (16 KB per unit, see
+                            // pack_weights_q8_kernel), or NULL; wscale[n] = scale of weight row n
   const float *wscale;
   const bf16 *wpacked;   // weights repacked by pack_weights_kernel (one contiguous 32 KB block per
                          // (tile, K block), in unit order); NULL: strided boxes through the W map
@@ -308,15 +308,17 @@ __global__ void row_scale_q8_kernel(const bf16 *__restrict__ W, int N, int K, fl
   m = warp_max(m);
   if (lane == 0) scale[n] = m > 0.f ? __fdiv_rn(m, 127.f) : 1.f;
 }
-// The codes in the GEMM's unit order: one 16 KB block per (tile, K block), 256 rows of 64 codes, rows
-// and tiles as in pack_weights_kernel (swiglu: 128 gate rows, then the 128 matching up rows). Rows and
-// columns past the matrix are zero.
+// The codes in the GEMM's unit order: one 16 KB block per (tile, K block), rows and tiles as in
+// pack_weights_kernel (swiglu: 128 gate rows, then the 128 matching up rows). A block is stored as
+// the expanding threads, one per weight row, read it: four planes of 16 codes, [plane][row][16 bytes],
+// and within a word of four codes the second and third are swapped, so that the pairs (0, 1) and
+// (2, 3) sit in bytes (0, 2) and (1, 3). Rows and columns past the matrix are zero.
 __global__ void pack_weights_q8_kernel(const bf16 *__restrict__ W, int N, int K, int tiles, int KB, int swiglu,
                                        int F, const float *__restrict__ scale, signed char *__restrict__ out) {
   const size_t total = (size_t)tiles * KB * BM * 4;                  // 16 codes per thread step
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(idx & 3), r = (int)((idx >> 2) & (BM - 1));
+    const int r = (int)(idx & (BM - 1)), c = (int)((idx >> 8) & 3);
     const size_t unit = idx >> 10;
     const int kb = (int)(unit % KB), tile = (int)(unit / KB);
     int n;
@@ -338,9 +340,10 @@ __global__ void pack_weights_q8_kernel(const bf16 *__restrict__ W, int N, int K,
         const float t = __fdiv_rn(__bfloat162float(W[(size_t)n * K + k]), s);
         q = (int)fminf(fmaxf(rintf(t), -127.f), 127.f);
       }
-      words[e >> 2] |= (uint32_t)(q & 0xff) << (8 * (e & 3));
+      const int byte = ((e & 1) << 1) | ((e >> 1) & 1);
+      words[e >> 2] |= (uint32_t)(q & 0xff) << (8 * byte);
     }
-    *reinterpret_cast<uint4 *>(out + unit * (BM * BK) + (size_t)r * BK + c * 16) = make_uint4(words[0], words[1], words[2], words[3]);
+    *reinterpret_cast<uint4 *>(out + unit * (BM * BK) + ((size_t)c * BM + r) * 16) = make_uint4(words[0], words[1], words[2], words[3]);
   }
 }
 

@@ -385,7 +385,7 @@ int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs
   ea.eps = ctx->desc.rms_eps;
   const bool prof = (ctx->prof_mask & ctx->phase) && 2 * (ctx->prof_used + 1) <= (int)ctx->prof_ev.size();
   if (prof) CU(cudaEventRecord(ctx->prof_ev[2 * ctx->prof_used], st));
-  const gemm_ck::RowPlan plan = gemm_ck::plan_rows(R, tiles, KB, ctx->fit);
+  const gemm_ck::RowPlan plan = gemm_ck::plan_rows(R, tiles, KB, ctx->fit, W.q8 != nullptr);
   const int chunks = plan.chunks, S = plan.S;
   ea.row0 = 0;
   ea.T = R;
@@ -398,7 +398,7 @@ int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs
     // start pulling the next matrix (up to L2_PREFETCH_BYTES of it)
     ea.pf_tiles = next_swiglu ? (next->N / 2 + 127) / 128 : (next->N + SV_TILE_ROWS - 1) / SV_TILE_ROWS;
     ea.pf_KB = (next->K + gemm_tc::BK - 1) / gemm_tc::BK;
-    ea.pf_S = gemm_ck::plan_rows(R, ea.pf_tiles, ea.pf_KB, ctx->fit).S;
+    ea.pf_S = gemm_ck::plan_rows(R, ea.pf_tiles, ea.pf_KB, ctx->fit, next->q8 != nullptr).S;
     ea.pf_unit_bytes = next->q8 ? gemm_tc::W_STAGE_BYTES / 2 : gemm_tc::W_STAGE_BYTES;
     const size_t per_cta = L2_PREFETCH_BYTES / ((size_t)ea.pf_tiles * ea.pf_S) / ea.pf_unit_bytes;
     ea.pf_units = per_cta < 1 ? 1 : (int)per_cta;
@@ -1852,7 +1852,7 @@ static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, i
   g_gemm_wait_ns = gemm_tc::WAIT_LIMIT_NS;           // the test hook holds for one call
   g_gemm_withhold = 0;
   const gemm_ck::ClusterFit fit = cluster_fit_of_current_device();
-  const gemm_ck::RowPlan plan = gemm_ck::plan_rows(T, tiles, KB, fit);
+  const gemm_ck::RowPlan plan = gemm_ck::plan_rows(T, tiles, KB, fit, false);
   ea.row0 = 0;
   ea.T = T;
   ea.chunk_rows = plan.chunk_rows;

@@ -1,0 +1,27 @@
+"""The int8 expansion at the row counts where its launches change: the last width of one MMA operand
+(64), the first launch of the long instantiation (65), its widest chunk (96) and the first launch of
+two chunks (97), against the quantised oracle."""
+import pytest
+
+from oracle import quant as Q
+from oracle.specvla import SpecVLAOracle, Tree
+from synth_inputs import configs as C, data
+
+import gpu_helpers as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_rows", [64, 65, 96, 97])
+def test_quantised_verify_at_chunk_edges(c0, n_rows):
+    desc = c0["desc"]
+    orc = SpecVLAOracle(C.TINY, Q.quantize_target(c0["weights"]))
+    gpu = G.make_gpu(desc, G.to_cuda(c0["weights"]), max_seq=256, max_episodes=1, max_rows=256, action_only=True,
+                     weight_bits=8)
+    tally = G.Tally()
+    ep, _, _ = G.prefill_both(orc, gpu, c0["embeds"].cuda(), c0["ids"], 0, tally, desc)
+    tok, par, dep = data.random_tree(n_rows, desc, seed=n_rows, max_depth=8, root_token=ep.root)
+    G.verify_both(orc, gpu, ep, Tree(tok, par, dep, [0.0] * n_rows), 40, tally, desc, where=f"q8.g(T={n_rows})")
+    # one wrong code would move a logit by about 1e-3; identical codes leave fp32 rounding only
+    assert tally.accepts == 1 and tally.caches == 1 and tally.max_logit_err < 2e-4, tally.max_logit_err
+    gpu.close()
