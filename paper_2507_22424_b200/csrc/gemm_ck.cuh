@@ -138,10 +138,15 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   constexpr int ROPE_ROWS = ROPE_SMEM ? 32 : 1, ROPE_HALF = ROPE_SMEM ? 64 : 1;
   __shared__ __align__(16) float2 s_rope[ROPE_ROWS * ROPE_HALF];
   __shared__ float s_red[8][MAX_T];
-  __shared__ int s_flag;
+  __shared__ int s_flag, s_fail;
   __shared__ float s_xv[4][2];             // EPI_TOPK: exchange between the two warps of a row group
   __shared__ int s_xi[4][2];
 
+  // a wait that gave up: for the host, and for this CTA's own way out
+  auto fail = [&](int code) {
+    atomicExch(err, code);
+    s_fail = 1;
+  };
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const int S = (int)cluster_size();
   const int rank = (int)cluster_rank();
@@ -161,13 +166,14 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int n_units = kb1 - kb0;
   const long long u0 = (long long)tile * KB + kb0;
   const int tiles = gridDim.x / S;
-  // rows of this CTA: one chunk. The 128-row instantiation takes its chunk length
-  // and MMA width from the launch (rows are spread evenly over the chunks of a long launch, so the
-  // width is rarely the full 128); the last chunk has a tensor map with its own box.
+  // rows of this CTA: one chunk. The 64- and 128-row instantiations take the MMA width, to the next
+  // eight rows, from the launch (a prefill of 34 rows: 3.25 -> 3.15 ms), the 128-row one its chunk
+  // length too (rows are spread evenly over the chunks of a long launch); the last chunk has a tensor
+  // map with its own box.
   const int row0 = ea.row0 + chunk * ea.chunk_rows;
   const int T = min(ea.T - chunk * ea.chunk_rows, ea.chunk_rows);
   const bool tail = chunk == (int)gridDim.y - 1;
-  const int tn = TN == MAX_T ? (tail ? ea.tn_tail : ea.tn_chunk) : TN;
+  const int tn = TN > 32 ? (tail ? ea.tn_tail : ea.tn_chunk) : TN;
   const CUtensorMap *xmap = (TN == MAX_T && tail) ? &tmXtail : &tmX;
   const uint32_t x_tx = (uint32_t)(2 * tn * BK * 2);
   const uint32_t stage_tx = Q8 ? (uint32_t)Q8_CODE_BYTES : W_STAGE_BYTES + x_tx;
@@ -210,6 +216,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     }
     mbar_init(tfull_bar, 1);
+    s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     grid_dep_launch();
@@ -251,7 +258,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     for (int it = npre, st = 0, ph = 0; it < n_units; it++) {
       const bool ok = mbar_wait(empty_bar(st), ph, ea.wait_ns);
       if (!__all_sync(0xffffffffu, ok)) {
-        if (lead) atomicExch(err, SV_ERR_WAIT_EMPTY);
+        if (lead) fail(SV_ERR_WAIT_EMPTY);
         break;
       }
       if (lead) {
@@ -273,7 +280,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     for (int it = 0, e = 0, ph = 1; it < n_units; it++) {
       const bool ok = it < NE || mbar_wait(efree_bar(e), ph, ea.wait_ns);
       if (!__all_sync(0xffffffffu, ok)) {
-        if (lead) atomicExch(err, SV_ERR_WAIT_EMPTY);
+        if (lead) fail(SV_ERR_WAIT_EMPTY);
         break;
       }
       if (lead) {
@@ -294,7 +301,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const bool ok = Q8 ? mbar_wait(xfull_bar(e), eph, ea.wait_ns) && mbar_wait(conv_bar(e), eph, ea.wait_ns)
                          : mbar_wait(full_bar(st), ph, ea.wait_ns);
       if (!__all_sync(0xffffffffu, ok)) {
-        if (lead) atomicExch(err, SV_ERR_WAIT_FULL);
+        if (lead) fail(SV_ERR_WAIT_FULL);
         break;
       }
       tc_fence_after();
@@ -407,7 +414,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (lane == 0) mbar_arrive(conv_bar(e));
         ok = __all_sync(0xffffffffu, got);
       }
-      if (!ok && lane == 0) atomicExch(err, SV_ERR_WAIT_FULL);
+      if (!ok && lane == 0) fail(SV_ERR_WAIT_FULL);
       __syncwarp();
       epi_barrier();
     }
@@ -418,7 +425,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       if (et == 0) {
         const bool done = mbar_wait(tfull_bar, 0, ea.wait_ns);
         s_flag = done ? 1 : 0;
-        if (!done) atomicExch(err, SV_ERR_WAIT_TMEM_FULL);
+        if (!done) fail(SV_ERR_WAIT_TMEM_FULL);
       }
       epi_barrier();
       have = s_flag != 0;
@@ -724,13 +731,15 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   }
   if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-  if (*reinterpret_cast<volatile int *>(err) != 0) {
-    const uint64_t t0 = global_ns();
-    while (global_ns() - t0 < 200000ull) __nanosleep(1000);
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // After a wait that gave up, copies may still be in flight: let them land. (The CTA's own flag and
+  // not *err: a load from global memory here is 0.4 us at the end of every launch.)
+  if (s_fail) {
+    const uint64_t t0 = global_ns();
+    while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+  }
   if (warp == 1) tc_dealloc(tmem_base, ck_tmem_cols(TN, Q8));
 }
 
@@ -835,7 +844,7 @@ inline int slices_for(int units, int KB, const ClusterFit &fit) {
 }
 
 // How a launch over R rows is cut: up to 128 rows are one chunk of the instantiation tn_of(R)
-// (between 65 and 128 rows: MMAs as wide as the rows need, to the next multiple of 8). Longer
+// (from 33 rows on with MMAs as wide as the rows need, to the next multiple of 8). Longer
 // launches (prefill, batched verification) are tensor-bound, and what counts is how evenly the
 // work fills the SMs: the rows are spread evenly over `chunks` chunks (grid y) of the 128-row
 // instantiation, and chunk count and K slices are chosen together by a cost estimate in SM
@@ -851,7 +860,7 @@ inline RowPlan plan_rows(int R, int tiles, int KB, const ClusterFit &fit, bool q
   const int max_rows = q8 ? Q8_MAX_T : MAX_T;
   RowPlan p = {1, MAX_T, tn_of(R), tn_of(R), 1};
   if (R <= max_rows) {
-    if (R > 64) p.tn_chunk = p.tn_tail = ceil8(R);
+    if (R > 32) p.tn_chunk = p.tn_tail = ceil8(R);
     p.S = slices_for(tiles, KB, fit);
     return p;
   }

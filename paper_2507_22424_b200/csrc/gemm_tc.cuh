@@ -37,11 +37,12 @@ constexpr int MAX_T = 128;
 
 __host__ __device__ constexpr int tn_of(int T) { return T <= 16 ? 16 : (T <= 32 ? 32 : (T <= 64 ? 64 : 128)); }
 __host__ __device__ constexpr int stage_bytes(int TN) { return W_STAGE_BYTES + 2 * TN * BK * 2; }
-// Up to 64 rows the ring leaves ~60 KB of the SM's shared memory free, so that the small kernels
-// between two GEMMs can be resident next to a GEMM CTA while it prefetches weights. At 128 rows
-// (prefill) a stage is 64 KB and two of them cannot cover the load latency: the ring takes a
-// third and most of the SM's shared memory.
-__host__ __device__ constexpr int stages_of(int TN) { return TN > 64 ? 3 : RING_BUDGET / stage_bytes(TN); }
+// Up to 32 rows the ring leaves ~60 KB of the SM's shared memory free, so that the small kernels
+// between two GEMMs can be resident next to a GEMM CTA while it prefetches weights (a fifth stage
+// measured the same). At 64 rows a stage is 48 KB and three of them do not cover the load latency:
+// four take a verification step of 64 rows from 3.77 to 3.59 ms, a prefill of 34 rows from 3.53 to
+// 3.35 ms. At 128 rows (prefill) a stage is 64 KB and three are what there is room for.
+__host__ __device__ constexpr int stages_of(int TN) { return TN > 64 ? 3 : TN > 32 ? 4 : RING_BUDGET / stage_bytes(TN); }
 __host__ __device__ constexpr int smem_bytes(int TN) { return stages_of(TN) * stage_bytes(TN) + 1024 + 256; }
 // Both limbs of X form ONE MMA operand (N = 2 TN: hi rows, then lo rows; 256 at most, the
 // largest N of an M = 128 MMA), which reads the weight operand from shared memory once for
