@@ -23,6 +23,7 @@
 #pragma once
 #include <cooperative_groups.h>
 #include "common.cuh"
+#include "gemm_tc.cuh"
 
 namespace attn {
 
@@ -30,6 +31,10 @@ constexpr int RB = 32;            // rows per block
 constexpr int KT = 32;            // key slots per tile
 constexpr int THREADS = 256;      // 8 warps x 4 rows
 constexpr int MAX_SPLITS = 8;         // key slices per row block = cluster size (8: the portable limit)
+// (32-row block, head) pairs up to which a launch takes the few-row kernel: up to 64 rows of 32 heads
+// its slices are what fills the SMs; at 96 rows it measured 21.7 us against 24 for 128-row blocks,
+// which one episode has 32 of, at 128 rows 23.3 against 22.5.
+constexpr int FEW_CTAS = 96;
 constexpr int MAX_SPLIT_CTAS = 148;   // CTAs of a launch that uses more than one key slice
 
 struct Args {
@@ -41,12 +46,14 @@ struct Args {
   float scale;
   bf16 *out;               // two limbs, [rows][H * DH] each
   size_t out_plane;
-  int splits;              // key slices per row block; the launch's cluster is (splits, 1, 1)
+  int splits;              // few-row launches: key slices per row block; the cluster is (splits, 1, 1)
+  unsigned long long wait_ns;   // long launches: limit of every mbarrier wait, and the status word
+  int *err;
 };
 
-__host__ __device__ inline int blocks_of(const EpArgs &ea) {
+__host__ __device__ inline int blocks_of(const EpArgs &ea, int rows) {
   int n = 0;
-  for (int i = 0; i < ea.n_ep; i++) n += (ea.nrows[i] + RB - 1) / RB;
+  for (int i = 0; i < ea.n_ep; i++) n += (ea.nrows[i] + rows - 1) / rows;
   return n;
 }
 // Shared memory: bf16 limb planes of Q [RB], K [KT], V [KT] (row pitch DH + 8: rows 16-byte
@@ -80,12 +87,9 @@ __device__ __forceinline__ void split4(const float4 v, uint2 &hi, uint2 &lo) {
   lo = make_uint2(*reinterpret_cast<const uint32_t *>(&l01), *reinterpret_cast<const uint32_t *>(&l23));
 }
 
-// SLICED: grid (row blocks x key slices, heads), cluster (slices, 1, 1): the few-row launches (a
-// verification step, a draft level). Unsliced (prefill: more CTAs than SMs): grid (heads, row
-// blocks), the blocks taken last to first: causal rows make the late blocks of an episode the long
-// ones, and CTAs are handed out x first, so every head's longest block starts before any short one
-// and the last wave is made of short blocks.
-template <int DH, bool SLICED>
+// The few-row launches (a verification step, a draft level): grid (row blocks x key slices, heads),
+// cluster (slices, 1, 1).
+template <int DH>
 __global__ void __launch_bounds__(THREADS, 1)
 tree_attention_kernel(const EpArgs ea, const Args a) {
   constexpr int PER = DH / 32;            // head-dim columns per lane in the slice merge
@@ -115,10 +119,10 @@ tree_attention_kernel(const EpArgs ea, const Args a) {
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int mb = warp & 1, wq = warp >> 1;         // 16-row block; key octet (scores) / head-dim quarter (sum)
-  const int h = SLICED ? blockIdx.y : blockIdx.x, hd = a.H * DH;
-  const int splits = SLICED ? a.splits : 1;
-  int bid = SLICED ? (int)blockIdx.x / splits : (int)gridDim.y - 1 - (int)blockIdx.y;
-  const int sp = SLICED ? (int)blockIdx.x - bid * splits : 0;
+  const int h = blockIdx.y, hd = a.H * DH;
+  const int splits = a.splits;
+  int bid = (int)blockIdx.x / splits;
+  const int sp = (int)blockIdx.x - bid * splits;
   int ei = 0;
   for (; ei < ea.n_ep; ei++) {
     const int nb = (ea.nrows[ei] + RB - 1) / RB;
@@ -342,27 +346,7 @@ tree_attention_kernel(const EpArgs ea, const Args a) {
   __syncthreads();
   const int ra = 16 * mb + (lane >> 2), rb = ra + 8;        // this thread's two rows
   const int cbase = (DH / 4) * wq + 2 * (lane & 3);          // + 8 nb: its column pairs
-  if (splits == 1) {
-    const float ia = 1.f / s_l[ra], ib = 1.f / s_l[rb];
-#pragma unroll
-    for (int nb = 0; nb < NB; nb++) {
-#pragma unroll
-      for (int half = 0; half < 2; half++) {
-        const int r = half ? rb : ra;
-        if (r >= nrows) continue;
-        const float inv = half ? ib : ia;
-        const float v0 = acc[nb][2 * half] * inv, v1 = acc[nb][2 * half + 1] * inv;
-        const size_t idx = (size_t)(row0 + r) * hd + h * DH + cbase + 8 * nb;
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
-        const float2 hf = __bfloat1622float2(hi);
-        *reinterpret_cast<__nv_bfloat162 *>(a.out + idx) = hi;
-        *reinterpret_cast<__nv_bfloat162 *>(a.out + a.out_plane + idx) = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
-      }
-    }
-    return;
-  }
-
-  // several key slices: leave this one in shared memory (over the query planes, which were
+  // leave this slice in shared memory (over the query planes, which were
   // only needed for the fragments), then merge rows sp, sp + splits, ... from all slices
   constexpr int LO = DH + 4;
   float *sO = reinterpret_cast<float *>(smem_raw);          // [RB][LO]: output, then max and sum
@@ -424,6 +408,457 @@ tree_attention_kernel(const EpArgs ea, const Args a) {
   // nobody leaves while a peer may still be reading its shared memory
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Launches with enough row blocks to fill the SMs without slicing keys (prefill, batched
+// verification): the two products on tcgen05.
+//
+// mma.sync runs at an eighth of the tcgen05 rate on this chip (23 clocks per m16n8k16 and scheduler
+// measured), and with three limb products per contraction it bounded these launches, whatever the
+// split of rows and keys over warps. Here a CTA takes 128 rows of one episode and one head:
+//   warps 0-3   own a row per thread: scores from TMEM, mask, online softmax, weights back to TMEM as
+//               the A operand of the second product (two limbs), rescaling of O when a maximum moved;
+//   warps 4-11  load K and V tiles of 64 slots (fp32, the next tile's loads in flight while this one
+//               is converted), split them into bf16 limbs and write them as swizzled K-major operands:
+//               K as [slot][dim], V transposed; two buffers. A thread transposes 8 slots x 4 dims of V;
+//               its four rows of V^T are DH / 4 apart, so that a warp's stores meet no bank twice: row
+//               j DH / 4 + i is dim 4 i + j, and so is column j DH / 4 + i of O;
+//   warp 12     issues the MMAs: S = Q K^T (hi hi in one accumulator, hi lo + lo hi in another, two
+//               buffers), O += P V (three products).
+// The scores of tile t + 1 are computed while the softmax of tile t runs. Arithmetic as in the few-row
+// kernel: 16 mantissa bits per operand, fp32 accumulation and softmax.
+// Per launch (32 heads of 128; the mma.sync kernel with one CTA per 32 rows before): 16 prefixes of
+// 296 rows 474 -> 219 us, one of 290 rows 27.4 -> 18.6 us, 8 trees of 27 rows against 290 slots 72 ->
+// 57 us. A tile takes 3500 clocks, bound by the softmax threads (about 2800) and the hand-overs; a
+// CTA spends another 5300 on queries and first tile and 3200 on its output.
+// Grid (heads, row blocks), the blocks taken last to first: causal rows make the late blocks of an
+// episode the long ones, and CTAs are handed out x first, so every head's longest block starts
+// before any short one.
+constexpr int TC_ROWS = 128, TC_KEYS = 64, TC_LOADERS = 256, TC_THREADS = 128 + TC_LOADERS + 32;
+template <int DH> __host__ __device__ constexpr int tc_q_bytes() { return TC_ROWS * DH * 2; }          // one limb
+template <int DH> __host__ __device__ constexpr int tc_kv_bytes() { return TC_KEYS * DH * 2; }         // one limb of K or of V
+template <int DH> __host__ __device__ constexpr int tc_smem_bytes() { return 2 * tc_q_bytes<DH>() + 8 * tc_kv_bytes<DH>() + 1024; }
+constexpr uint32_t TC_S = 0, TC_P = 256, TC_O = 320;       // TMEM columns: S [2][main 64 | cross 64], P hi | lo, O
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void st_shared16(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+// eight floats -> 16 bytes of hi limbs and 16 bytes of lo limbs
+__device__ __forceinline__ void store_split8(uint32_t hi_addr, uint32_t lo_addr, const float (&v)[8]) {
+  uint2 h0, l0, h1, l1;
+  split4(make_float4(v[0], v[1], v[2], v[3]), h0, l0);
+  split4(make_float4(v[4], v[5], v[6], v[7]), h1, l1);
+  st_shared16(hi_addr, h0.x, h0.y, h1.x, h1.y);
+  st_shared16(lo_addr, l0.x, l0.y, l1.x, l1.y);
+}
+
+template <int DH>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+row_attention_kernel(const EpArgs ea, const Args a) {
+  using namespace gemm_tc;
+  constexpr int QB = tc_q_bytes<DH>(), KVB = tc_kv_bytes<DH>();
+  constexpr int C8 = DH / 8;                       // 16-byte chunks (8 dims) per row
+  constexpr int C4 = DH / 4;                       // float4 per row
+  constexpr int NKC = TC_KEYS * C8 / TC_LOADERS;   // K chunks per loader thread and tile
+  static_assert((TC_KEYS / 8) * C4 <= TC_LOADERS, "one 8 x 4 piece of V per loader thread");
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  // Q hi | Q lo | per buffer: K hi | K lo | V^T hi | V^T lo
+  auto kv_base = [&](int b) { return base + (uint32_t)(2 * QB + b * 4 * KVB); };
+  __shared__ __align__(8) unsigned long long s_bar[10];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_fail;
+  const uint32_t bars = smem_u32(s_bar);
+  auto k_full = [&](int b) { return bars + 8u * b; };           // the loaders have written K (V) of buffer b
+  auto v_full = [&](int b) { return bars + 8u * (2 + b); };
+  auto s_full = [&](int b) { return bars + 8u * (4 + b); };     // scores are in S buffer b, K of buffer b is free
+  auto v_free = [&](int b) { return bars + 8u * (6 + b); };     // V of buffer b is free
+  const uint32_t p_full = bars + 8u * 8, o_full = bars + 8u * 9;   // weights are in TMEM / O includes their tile
+
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  if (tid == 0) {
+    for (int b = 0; b < 2; b++) {
+      mbar_init(k_full(b), TC_LOADERS / 32);
+      mbar_init(v_full(b), TC_LOADERS / 32);
+      mbar_init(v_free(b), 1);
+      mbar_init(s_full(b), 1);
+    }
+    mbar_init(p_full, 4);
+    mbar_init(o_full, 1);
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 12) {
+    tc_alloc(smem_u32(&s_tmem), 512);
+    tc_relinquish();
+  }
+  pdl_wait();
+
+  const int h = blockIdx.x, hd = a.H * DH;
+  int bid = (int)gridDim.y - 1 - (int)blockIdx.y, ei = 0;
+  for (; ei + 1 < ea.n_ep; ei++) {
+    const int nb = (ea.nrows[ei] + TC_ROWS - 1) / TC_ROWS;
+    if (bid < nb) break;
+    bid -= nb;
+  }
+  const int row0 = ea.row0[ei] + bid * TC_ROWS;
+  const int nrows = min(TC_ROWS, ea.nrows[ei] - bid * TC_ROWS);
+  const float *kbase = a.cache + (size_t)ea.eps[ei] * a.ep_stride + (size_t)h * DH;
+  const float *vbase = kbase + (size_t)a.max_seq * hd;
+
+  // last slot that any row sees: every warp finds it for itself
+  int kmax = 0;
+  {
+    int vis[TC_ROWS / 32], at[TC_ROWS / 32];
+    uint4 m[TC_ROWS / 32];
+#pragma unroll
+    for (int k = 0; k < TC_ROWS / 32; k++) {               // (all loads first)
+      const int r = row0 + min(lane + 32 * k, nrows - 1);
+      vis[k] = a.rt.nvis[r];
+      at[k] = a.rt.tbase[r];
+      m[k] = *reinterpret_cast<const uint4 *>(a.rt.mask + (size_t)r * 4);
+    }
+#pragma unroll
+    for (int k = 0; k < TC_ROWS / 32; k++) {
+      const int last = m[k].w ? 128 - __clz(m[k].w) : m[k].z ? 96 - __clz(m[k].z) : m[k].y ? 64 - __clz(m[k].y)
+                       : m[k].x ? 32 - __clz(m[k].x) : 0;
+      kmax = max(kmax, max(vis[k], last ? at[k] + last : 0));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+  kmax = min(kmax, a.max_seq);
+  const int tiles = (kmax + TC_KEYS - 1) / TC_KEYS;
+
+  // the loaders' first tile is on its way while the others prepare the queries
+  const int lt = tid - 128;
+  const int vg = lt / C4, vd = lt % C4;                     // V: this thread's slot group and float4 of dims
+  float4 kr[NKC][2], vr[8];
+  auto load_k = [&](int t) {
+#pragma unroll
+    for (int k = 0; k < NKC; k++) {
+      const int i = lt + k * TC_LOADERS, slot = t * TC_KEYS + i / C8;
+      kr[k][0] = kr[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (slot < kmax) {
+        const float4 *p = reinterpret_cast<const float4 *>(kbase + (size_t)slot * hd + (i % C8) * 8);
+        kr[k][0] = p[0];
+        kr[k][1] = p[1];
+      }
+    }
+  };
+  auto load_v = [&](int t) {
+    const float *p = vbase + (size_t)(t * TC_KEYS + vg * 8) * hd + vd * 4;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      vr[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (vg < TC_KEYS / 8 && t * TC_KEYS + vg * 8 + j < kmax) vr[j] = *reinterpret_cast<const float4 *>(p + (size_t)j * hd);
+    }
+  };
+  const bool loader = warp >= 4 && warp < 12;
+  if (loader && tiles > 0) {
+    load_k(0);
+    load_v(0);
+  }
+  // what this thread's row sees (warps 0-3): slots [0, nv) and bits of a 128-bit mask from slot tb on
+  int nv = 0, tb = 0;
+  unsigned long long mlo = 0, mhi = 0;
+  if (warp < 4) {
+    if (tid < nrows) {
+      const int r = row0 + tid;
+      nv = a.rt.nvis[r];
+      tb = a.rt.tbase[r];
+      const uint4 m = *reinterpret_cast<const uint4 *>(a.rt.mask + (size_t)r * 4);
+      mlo = m.x | ((unsigned long long)m.y << 32);
+      mhi = m.z | ((unsigned long long)m.w << 32);
+    }
+  }
+  // the query rows, scaled, as limbs (rows past nrows are zero): blocks of 64 dims, 128-byte rows
+  if (warp < 12) {
+    constexpr int QT = 128 + TC_LOADERS, NQ = (TC_ROWS * C8 + QT - 1) / QT;
+    float4 x[NQ][2];
+#pragma unroll
+    for (int k = 0; k < NQ; k++) {
+      const int i = tid + k * QT, r = i / C8;
+      x[k][0] = x[k][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < nrows) {
+        const float4 *p = reinterpret_cast<const float4 *>(a.q + (size_t)(row0 + r) * hd + h * DH + (i % C8) * 8);
+        x[k][0] = p[0];
+        x[k][1] = p[1];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NQ; k++) {
+      const int i = tid + k * QT, r = i / C8, c = i % C8;
+      if (r >= TC_ROWS) break;
+      const uint32_t at = base + (uint32_t)((c >> 3) * (TC_ROWS * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+      const float v[8] = {x[k][0].x * a.scale, x[k][0].y * a.scale, x[k][0].z * a.scale, x[k][0].w * a.scale,
+                          x[k][1].x * a.scale, x[k][1].y * a.scale, x[k][1].z * a.scale, x[k][1].w * a.scale};
+      store_split8(at, at + QB, v);
+    }
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  auto fail = [&](int code) {
+    atomicExch(a.err, code);
+    s_fail = 1;
+  };
+
+  if (loader) {
+    // ------------------------------------------------------------------ loaders
+    for (int t = 0; t < tiles; t++) {
+      const int b = t & 1;
+      bool ok = t < 2 || mbar_wait(s_full(b), ((t >> 1) - 1) & 1, a.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0) fail(SV_ERR_WAIT_EMPTY);
+        break;
+      }
+      const uint32_t kb = kv_base(b);
+#pragma unroll
+      for (int k = 0; k < NKC; k++) {
+        const int i = lt + k * TC_LOADERS, key = i / C8, c = i % C8;
+        const uint32_t at = kb + (uint32_t)((c >> 3) * (TC_KEYS * 128) + key * 128 + (((c & 7) ^ (key & 7)) << 4));
+        const float v[8] = {kr[k][0].x, kr[k][0].y, kr[k][0].z, kr[k][0].w, kr[k][1].x, kr[k][1].y, kr[k][1].z, kr[k][1].w};
+        store_split8(at, at + KVB, v);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(k_full(b));
+      if (t + 1 < tiles) load_k(t + 1);
+      ok = t < 2 || mbar_wait(v_free(b), ((t >> 1) - 1) & 1, a.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0) fail(SV_ERR_WAIT_EMPTY);
+        break;
+      }
+      if (vg < TC_KEYS / 8) {
+        const float v[4][8] = {{vr[0].x, vr[1].x, vr[2].x, vr[3].x, vr[4].x, vr[5].x, vr[6].x, vr[7].x},
+                               {vr[0].y, vr[1].y, vr[2].y, vr[3].y, vr[4].y, vr[5].y, vr[6].y, vr[7].y},
+                               {vr[0].z, vr[1].z, vr[2].z, vr[3].z, vr[4].z, vr[5].z, vr[6].z, vr[7].z},
+                               {vr[0].w, vr[1].w, vr[2].w, vr[3].w, vr[4].w, vr[5].w, vr[6].w, vr[7].w}};
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          const int r = j * C4 + vd;
+          const uint32_t at = kb + (uint32_t)(2 * KVB + r * 128 + ((vg ^ (r & 7)) << 4));
+          store_split8(at, at + KVB, v[j]);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(v_full(b));
+      if (t + 1 < tiles) load_v(t + 1);
+    }
+  } else if (warp == 12) {
+    // ------------------------------------------------------------------ MMA issuer
+    const bool lead = elect_one();
+    constexpr uint32_t idesc_s = instr_desc(TC_KEYS), idesc_o = instr_desc(DH);
+    auto scores = [&](int t) {
+      const int b = t & 1;
+      const bool ok = mbar_wait(k_full(b), (t >> 1) & 1, a.wait_ns);
+      if (!__all_sync(0xffffffffu, ok)) return false;
+      tc_fence_after();
+      const uint64_t qh = smem_desc(base), ql = smem_desc(base + QB);
+      const uint64_t kh = smem_desc(kv_base(b)), kl = smem_desc(kv_base(b) + KVB);
+      const uint32_t s0 = tmem + TC_S + (uint32_t)(b * 128), s1 = s0 + 64;
+      if (lead) {
+#pragma unroll
+        for (int ks = 0; ks < DH / 16; ks++) {
+          const uint64_t qo = (uint64_t)(((ks >> 2) * (TC_ROWS * 128) + (ks & 3) * 32) >> 4);
+          const uint64_t ko = (uint64_t)(((ks >> 2) * (TC_KEYS * 128) + (ks & 3) * 32) >> 4);
+          tc_mma(s0, qh + qo, kh + ko, idesc_s, ks > 0 ? 1u : 0u);
+          tc_mma(s1, qh + qo, kl + ko, idesc_s, ks > 0 ? 1u : 0u);
+          tc_mma(s1, ql + qo, kh + ko, idesc_s, 1u);
+        }
+        tc_commit(s_full(b));
+      }
+      __syncwarp();
+      return true;
+    };
+    bool ok = tiles == 0 || scores(0);
+    for (int t = 0; ok && t < tiles; t++) {
+      // whichever comes first: the next tile's keys (its S buffer was read before the weights of tile
+      // t - 1 were reported), or this tile's weights
+      bool next_done = t + 1 >= tiles;
+      uint64_t t0 = 0;
+      for (int spin = 0;; spin++) {
+        if (!next_done && __all_sync(0xffffffffu, mbar_test(k_full((t + 1) & 1), ((t + 1) >> 1) & 1))) {
+          ok = scores(t + 1);
+          next_done = true;
+        }
+        if (!ok || __all_sync(0xffffffffu, mbar_test(p_full, t & 1))) break;
+        if ((spin & 1023) == 1023) {
+          const uint64_t now = global_ns();
+          if (t0 == 0) t0 = now;
+          ok = __all_sync(0xffffffffu, now - t0 <= a.wait_ns);
+        }
+      }
+      if (!ok) break;
+      ok = mbar_wait(v_full(t & 1), (t >> 1) & 1, a.wait_ns);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t vb = kv_base(t & 1) + 2 * KVB;
+      const uint64_t vh = smem_desc(vb), vl = smem_desc(vb + KVB);
+      const uint32_t ph = tmem + TC_P, pl = ph + 32, o = tmem + TC_O;
+      if (lead) {
+#pragma unroll
+        for (int ks = 0; ks < TC_KEYS / 16; ks++) {
+          const uint64_t vo = (uint64_t)((ks * 32) >> 4);
+          tc_mma_ta(o, ph + ks * 8, vh + vo, idesc_o, (t > 0 || ks > 0) ? 1u : 0u);
+          tc_mma_ta(o, ph + ks * 8, vl + vo, idesc_o, 1u);
+          tc_mma_ta(o, pl + ks * 8, vh + vo, idesc_o, 1u);
+        }
+        tc_commit(v_free(t & 1));
+        tc_commit(o_full);
+      }
+      __syncwarp();
+      if (!next_done) ok = scores(t + 1);
+    }
+    if (!ok && lead) fail(SV_ERR_WAIT_FULL);
+    __syncwarp();
+  } else if (warp < 4) {
+    // ------------------------------------------------------------------ softmax: row tid
+    const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+    float m = -INFINITY, l = 0.f;
+    bool ok = true;
+    for (int t = 0; t < tiles; t++) {
+      ok = mbar_wait(s_full(t & 1), (t >> 1) & 1, a.wait_ns);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      float s[TC_KEYS];
+#pragma unroll
+      for (int c = 0; c < TC_KEYS; c += 32) {
+        uint32_t x[32], y[32];
+        tmem_ld32(tl + TC_S + (uint32_t)((t & 1) * 128 + c), x);
+        tmem_ld32(tl + TC_S + (uint32_t)((t & 1) * 128 + 64 + c), y);
+        tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; j++) s[c + j] = __uint_as_float(x[j]) + __uint_as_float(y[j]);
+      }
+      // which of the tile's slots the row sees
+      const int p = nv - t * TC_KEYS, off = tb - t * TC_KEYS;
+      unsigned long long vis = p >= 64 ? ~0ull : p > 0 ? (1ull << p) - 1ull : 0ull;
+      if (off >= 0) {
+        if (off < 64) vis |= mlo << off;
+      } else if (off > -64) {
+        vis |= (mlo >> -off) | (mhi << (64 + off));
+      } else if (off > -128) {
+        vis |= mhi >> (-off - 64);
+      }
+      if (!__all_sync(0xffffffffu, vis == ~0ull)) {
+        const uint32_t v0 = (uint32_t)vis, v1 = (uint32_t)(vis >> 32);
+#pragma unroll
+        for (int j = 0; j < 32; j++) {
+          if (!((v0 >> j) & 1u)) s[j] = -INFINITY;
+          if (!((v1 >> j) & 1u)) s[32 + j] = -INFINITY;
+        }
+      }
+      float mx[4] = {m, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int j = 0; j < TC_KEYS; j++) mx[j & 3] = fmaxf(mx[j & 3], s[j]);
+      const float mn = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+      const float z = mn == -INFINITY ? 0.f : mn;            // (a row that has seen nothing yet: weights of zero)
+      const float corr = mn == -INFINITY ? 1.f : __expf(m - mn);
+      const bool moved = __any_sync(0xffffffffu, mn != m);
+      m = mn;
+      float ps[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t hi[32], lo[32];
+#pragma unroll
+      for (int j = 0; j < TC_KEYS; j += 4) {
+        const float4 e = make_float4(__expf(s[j] - z), __expf(s[j + 1] - z), __expf(s[j + 2] - z), __expf(s[j + 3] - z));
+        ps[0] += e.x; ps[1] += e.y; ps[2] += e.z; ps[3] += e.w;
+        uint2 eh, el;
+        split4(e, eh, el);
+        hi[j / 2] = eh.x; hi[j / 2 + 1] = eh.y;
+        lo[j / 2] = el.x; lo[j / 2 + 1] = el.y;
+      }
+      l = l * corr + ((ps[0] + ps[1]) + (ps[2] + ps[3]));
+      if (t > 0) {
+        // the previous tile's product has read the weights and written O
+        ok = mbar_wait(o_full, (t - 1) & 1, a.wait_ns);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        if (moved) {
+#pragma unroll 1
+          for (int c = 0; c < DH; c += 32) {
+            uint32_t o[32];
+            tmem_ld32(tl + TC_O + c, o);
+            tc_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 32; j++) o[j] = __float_as_uint(__uint_as_float(o[j]) * corr);
+            tc_st32(tl + TC_O + c, o);
+          }
+        }
+      }
+      tc_st32(tl + TC_P, hi);
+      tc_st32(tl + TC_P + 32, lo);
+      tc_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full);
+    }
+    if (ok && tiles > 0) {
+      ok = mbar_wait(o_full, (tiles - 1) & 1, a.wait_ns);
+      ok = __all_sync(0xffffffffu, ok);
+      tc_fence_after();
+    }
+    if (!ok && lane == 0) fail(SV_ERR_WAIT_TMEM_FULL);
+    // output limbs, through the query planes (every product has been computed): rows of DH + 8 elements
+    constexpr int LD = DH + 8;
+    bf16 *oh = reinterpret_cast<bf16 *>(smem_raw + (base - smem_u32(smem_raw))) + warp * 32 * LD;
+    bf16 *ol = oh + TC_ROWS * LD;
+    const float inv = 1.f / l;
+    if (ok) {
+#pragma unroll 1
+      for (int c = 0; c < C4; c += 8) {                    // dims 4 c .. 4 c + 31: eight columns of each quarter
+        uint32_t o0[8], o1[8], o2[8], o3[8];
+        tc_ld8(tl + TC_O + c, o0);
+        tc_ld8(tl + TC_O + C4 + c, o1);
+        tc_ld8(tl + TC_O + 2 * C4 + c, o2);
+        tc_ld8(tl + TC_O + 3 * C4 + c, o3);
+        tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          uint2 eh, el;
+          split4(make_float4(__uint_as_float(o0[j]) * inv, __uint_as_float(o1[j]) * inv, __uint_as_float(o2[j]) * inv,
+                             __uint_as_float(o3[j]) * inv), eh, el);
+          *reinterpret_cast<uint2 *>(oh + lane * LD + 4 * (c + j)) = eh;
+          *reinterpret_cast<uint2 *>(ol + lane * LD + 4 * (c + j)) = el;
+        }
+      }
+      __syncwarp();
+      for (int i = lane; i < 32 * C8; i += 32) {
+        const int r = warp * 32 + i / C8, c = (i % C8) * 8;
+        if (r >= nrows) break;
+        const size_t idx = (size_t)(row0 + r) * hd + h * DH + c;
+        *reinterpret_cast<uint4 *>(a.out + idx) = *reinterpret_cast<const uint4 *>(oh + (i / C8) * LD + c);
+        *reinterpret_cast<uint4 *>(a.out + a.out_plane + idx) = *reinterpret_cast<const uint4 *>(ol + (i / C8) * LD + c);
+      }
+    }
+    tc_fence_before();
+  }
+  pdl_launch();
+  __syncthreads();
+  tc_fence_after();
+  if (s_fail) {
+    const uint64_t t0 = global_ns();
+    while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+  }
+  if (warp == 12) tc_dealloc(tmem, 512);
 }
 
 }  // namespace attn

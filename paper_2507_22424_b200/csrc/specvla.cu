@@ -464,35 +464,30 @@ int attention(specvla_ctx *ctx, const EpArgs &rows, const float *cache, size_t e
   a.scale = 1.f / sqrtf((float)d.head_dim);
   a.out = ctx->ao.p;
   a.out_plane = ctx->ao.plane;
-  const int blocks = attn::blocks_of(rows);
+  a.wait_ns = ctx->wait_ns;
+  a.err = ctx->err;
+  const int blocks = attn::blocks_of(rows, attn::RB);
   if (blocks < 1) return SPECVLA_OK;
-  // few row blocks: slice the key range so that the launch still covers the SMs
   const int ctas = blocks * d.n_heads;
-  a.splits = 1;
-  if (ctas < 96) {
-    a.splits = attn::MAX_SPLIT_CTAS / ctas;
-    if (a.splits > attn::MAX_SPLITS) a.splits = attn::MAX_SPLITS;
-    if (a.splits < 1) a.splits = 1;
-  }
-  // the key slices of a row block are one cluster (they merge through distributed shared memory)
-  // (unsliced: heads on x, see the kernel)
-  const dim3 grid = a.splits == 1 ? dim3(d.n_heads, blocks) : dim3(blocks * a.splits, d.n_heads);
   cudaLaunchAttribute at[2];
-  cudaLaunchConfig_t cfg = launch_cfg(grid, dim3(attn::THREADS), st, &at[0], ctx->use_pdl);
-  at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-  at[cfg.numAttrs].val.clusterDim.x = a.splits;
-  at[cfg.numAttrs].val.clusterDim.y = 1;
-  at[cfg.numAttrs].val.clusterDim.z = 1;
-  cfg.numAttrs++;
-  const bool sliced = a.splits > 1;
-  if (d.head_dim == 128) {
-    cfg.dynamicSmemBytes = attn::smem_bytes<128>();
-    CU(sliced ? cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<128, true>, rows, a)
-              : cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<128, false>, rows, a));
+  if (ctas <= attn::FEW_CTAS) {
+    // the slices of a row block are one cluster (they merge through distributed shared memory)
+    a.splits = std::max(1, std::min(attn::MAX_SPLIT_CTAS / ctas, attn::MAX_SPLITS));
+    cudaLaunchConfig_t cfg = launch_cfg(dim3(blocks * a.splits, d.n_heads), dim3(attn::THREADS), st, &at[0], ctx->use_pdl);
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = a.splits;
+    at[cfg.numAttrs].val.clusterDim.y = 1;
+    at[cfg.numAttrs].val.clusterDim.z = 1;
+    cfg.numAttrs++;
+    cfg.dynamicSmemBytes = d.head_dim == 128 ? attn::smem_bytes<128>() : attn::smem_bytes<64>();
+    CU(d.head_dim == 128 ? cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<128>, rows, a)
+                         : cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<64>, rows, a));
   } else {
-    cfg.dynamicSmemBytes = attn::smem_bytes<64>();
-    CU(sliced ? cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<64, true>, rows, a)
-              : cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<64, false>, rows, a));
+    cudaLaunchConfig_t cfg = launch_cfg(dim3(d.n_heads, attn::blocks_of(rows, attn::TC_ROWS)), dim3(attn::TC_THREADS), st,
+                                        &at[0], ctx->use_pdl);
+    cfg.dynamicSmemBytes = d.head_dim == 128 ? attn::tc_smem_bytes<128>() : attn::tc_smem_bytes<64>();
+    CU(d.head_dim == 128 ? cudaLaunchKernelEx(&cfg, attn::row_attention_kernel<128>, rows, a)
+                         : cudaLaunchKernelEx(&cfg, attn::row_attention_kernel<64>, rows, a));
   }
   ctx->launches++;
   return SPECVLA_OK;
@@ -968,14 +963,11 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   cudaMemsetAsync(ctx->st, 0, sizeof(EpState) * desc->max_episodes);
   cudaMemsetAsync(ctx->trees, 0, sizeof(DevTree) * desc->max_episodes);
   cudaMemsetAsync(ctx->err, 0, 32 * sizeof(int));
-  cudaFuncSetAttribute(attn::tree_attention_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       attn::smem_bytes<128>());
-  cudaFuncSetAttribute(attn::tree_attention_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       attn::smem_bytes<128>());
-  cudaFuncSetAttribute(attn::tree_attention_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       attn::smem_bytes<64>());
-  cudaFuncSetAttribute(attn::tree_attention_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       attn::smem_bytes<64>());
+  auto smem_of = [](auto kernel, int bytes) { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  smem_of(attn::tree_attention_kernel<128>, attn::smem_bytes<128>());
+  smem_of(attn::tree_attention_kernel<64>, attn::smem_bytes<64>());
+  smem_of(attn::row_attention_kernel<128>, attn::tc_smem_bytes<128>());
+  smem_of(attn::row_attention_kernel<64>, attn::tc_smem_bytes<64>());
   if (cudaDeviceSynchronize() != cudaSuccess || !pack_ok) {
     cudaFreeHost(ctx->pinned);
     delete ctx;

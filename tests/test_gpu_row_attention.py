@@ -1,0 +1,57 @@
+"""Attention of launches with many row blocks (batched prefill, batched verification) against the same
+episodes taken one at a time, whose few-row kernel the oracle tests pin; one episode against the
+oracle itself. Row counts sit at the edges of the 32- and 64-row blocks and of the 32-key tiles;
+the episode counts give launches of 32-row and of 64-row blocks."""
+import random
+
+import pytest
+import torch
+
+from oracle.specvla import SpecVLAOracle
+from synth_inputs import configs as C, data
+
+import gpu_helpers as G
+
+pytestmark = pytest.mark.gpu
+
+DESCS = [C.ModelDesc(n_layers=2, d_model=8 * hd, n_heads=8, head_dim=hd, d_ffn=688, vocab=1024, action_base=768)
+         for hd in (64, 128)]
+
+
+@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
+@pytest.mark.parametrize("n_ep", [16, 60])
+def test_batched_rows_equal_single_episodes(desc, n_ep):
+    w = data.make_weights(desc, 31)
+    rng = random.Random(n_ep)
+    edges = [65, 31, 97, 64, 33, 128, 96, 129, 63, 127]
+    lens = [edges[i % len(edges)] if n_ep == 60 or i % 2 == 0 else 70 + i for i in range(n_ep)]
+    ids = [[rng.randrange(desc.action_base) for _ in range(n)] for n in lens]
+    gpu = G.make_gpu(desc, G.to_cuda(w), max_seq=320, max_episodes=n_ep, max_rows=sum(lens), action_only=True)
+    embeds = torch.zeros(sum(lens), desc.d_model, dtype=torch.bfloat16, device="cuda")
+    eps = list(range(n_ep))
+    trees = []
+    for e in eps:
+        tok, par, dep = data.random_tree([27, 40, 65][e % 3], desc, seed=e, max_depth=8, root_token=None)
+        trees.append(dict(tokens=[desc.action_base + e] + list(tok)[1:], parent=list(par), depth=list(dep)))
+    first, logits = gpu.prefill(eps, embeds, sum(ids, []), lens, want_logits=True)
+    greedy = gpu.score_tree(eps, trees)
+    margin = gpu.read_buffer(2, len(greedy), torch.float32)
+    r0, checked = 0, 0
+    for e in eps:
+        f1, l1 = gpu.prefill([e], embeds[:lens[e]], ids[e], [lens[e]], want_logits=True)
+        # both paths carry 16 mantissa bits per operand: 2 layers, logits of order 1
+        assert (logits[e] - l1[0]).abs().max() < 1e-4, (e, lens[e])
+        g1 = gpu.score_tree([e], [trees[e]])
+        m1 = gpu.read_buffer(2, len(g1), torch.float32)
+        for i, (a, b) in enumerate(zip(greedy[r0:r0 + len(g1)], g1)):
+            if float(m1[i]) > 1e-3:
+                assert a == b and abs(float(margin[r0 + i] - m1[i])) < 1e-3, (e, i)
+                checked += 1
+        r0 += len(g1)
+    assert checked > 0.9 * len(greedy)
+    orc = SpecVLAOracle(desc, w)
+    for e in (1, 7):
+        embeds_e, ids_e = torch.zeros(lens[e], desc.d_model, dtype=torch.bfloat16), torch.tensor(ids[e])
+        _, ref, _ = orc.prefill(embeds_e, ids_e, want_logits=True)
+        assert (logits[e].cpu().double() - ref.reshape(-1)).abs().max() < 1e-3, (e, lens[e])
+    gpu.close()
