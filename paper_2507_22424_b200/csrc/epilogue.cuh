@@ -16,12 +16,6 @@ namespace epi {
 
 constexpr int THREADS = 256;
 
-__device__ __forceinline__ void store2(bf16 *hi_plane, size_t plane, size_t idx, float v) {
-  const bf16 hi = __float2bfloat16(v);
-  hi_plane[idx] = hi;
-  hi_plane[plane + idx] = __float2bfloat16(v - __bfloat162float(hi));
-}
-
 __device__ __forceinline__ float block_sum(float v, float *red) {
   v = warp_sum(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -113,10 +107,20 @@ __global__ void features_kernel(const float *__restrict__ x, const float *__rest
   }
 }
 
-// Two-limb split of an fp32 matrix (stand-alone GEMM entry point).
-__global__ void split_limbs_kernel(const float *__restrict__ x, size_t n, bf16 *__restrict__ out) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) store2(out, n, i, x[i]);
+// Two-limb split of an fp32 matrix (stand-alone GEMM entry point), four values a thread (n is a
+// multiple of 8; VEC: x starts on 16 bytes), and zeroes for the GEMM's status words. The GEMM may
+// start, and fill its ring with weights, while this kernel runs.
+template <bool VEC>
+__global__ void __launch_bounds__(THREADS)
+split_limbs_kernel(const float *__restrict__ x, size_t n, bf16 *__restrict__ out, int *__restrict__ status,
+                   int n_status) {
+  pdl_launch();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n_status; i += THREADS) status[i] = 0;
+  const size_t i = ((size_t)blockIdx.x * THREADS + threadIdx.x) * 4;
+  if (i >= n) return;
+  const float4 v = VEC ? *reinterpret_cast<const float4 *>(x + i) : make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  store_limbs4(out, n, i, v);
 }
 
 using sv::Top2;
