@@ -101,6 +101,7 @@ struct specvla_ctx {
   XBuf xn, xin, ao, hid, lm_in;
   int *err;                     // device status word written by bounded waits that gave up
   RowTable rt;
+  int *tok_in;                  // token ids of the prefill in flight
   int *feat_src, *lm_rows, *greedy, *top_tok, *out_m, *out_tok, *out_path;
   EpState *st;
   DevTree *trees;
@@ -124,7 +125,7 @@ struct specvla_ctx {
   size_t pinned_bytes;
   int *pin_small;               // 4096 ints of results read back
   DevTree *pin_trees;           // max_episodes trees
-  int *pin_rows;                // 11 * max_rows + SV_MAX_EP ints: row tables of the target and of the draft model
+  int *pin_rows;                // max_rows ints: token ids of a prefill
   std::vector<int> hP, hPending;  // host mirror of P and n_pending; -1 = not prefilled
   std::vector<int> hTreeRows;     // rows of the device-resident tree left by the last draft call
   int last_rows;                // rows of the last target forward
@@ -138,7 +139,8 @@ struct specvla_ctx {
   bool use_device_loop;
   bool loop_unavailable;          // capturing or instantiating the loop graph failed once: the host runs the loop
   ChunkState *chunk;              // device
-  ChunkState *pin_chunk;          // pinned copy read back after the loop, then max_episodes EpState
+  ChunkState *pin_chunk;          // pinned copy of what is read back after the loop: chunk, st and err as they
+  size_t chunk_span;              // lie in the workspace
   cudaStream_t cap_stream;        // capture happens on a stream of the context's own
   cudaGraph_t loop_graph;
   cudaGraphExec_t loop_exec;
@@ -301,10 +303,12 @@ size_t carve(specvla_ctx *c, char *base) {
   c->out_m = cv.take<int>(E);
   c->out_tok = cv.take<int>(E * (SV_MAX_DEPTH + 1));
   c->out_path = cv.take<int>(E * (SV_MAX_DEPTH + 1));
-  c->st = cv.take<EpState>(E);
   c->trees = cv.take<DevTree>(E);
-  c->err = cv.take<int>(32);
+  c->tok_in = cv.take<int>(R);
+  // (read back together after a chunk: one copy)
   c->chunk = cv.take<ChunkState>(1);
+  c->st = cv.take<EpState>(E);
+  c->err = cv.take<int>(32);
   // persistent forward kernel: packed operands, partial tiles, attention slices, candidates
   if (pk_shapes_ok(d) && d.weight_bits != 8) {
     const size_t G = c->pk_G;
@@ -935,8 +939,9 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   ctx->hTreeRows.assign(desc->max_episodes, 0);
   const size_t small_b = 4096 * sizeof(int);
   const size_t trees_b = (sizeof(DevTree) * desc->max_episodes + 255) / 256 * 256;
-  const size_t rows_b = ((size_t)desc->max_rows * 11 + SV_MAX_EP + 256) * sizeof(int);
-  ctx->pinned_bytes = small_b + trees_b + rows_b + sizeof(ChunkState) + sizeof(EpState) * desc->max_episodes;
+  const size_t rows_b = ((size_t)desc->max_rows * sizeof(int) + 255) / 256 * 256;
+  ctx->chunk_span = reinterpret_cast<char *>(ctx->err + 1) - reinterpret_cast<char *>(ctx->chunk);
+  ctx->pinned_bytes = small_b + trees_b + rows_b + ctx->chunk_span;
   ctx->cuda_err[0] = 0;
   if (cudaHostAlloc(&ctx->pinned, ctx->pinned_bytes, cudaHostAllocDefault) != cudaSuccess) {
     delete ctx;
@@ -1071,36 +1076,17 @@ static int prefill_enqueue(specvla_ctx *ctx, int n_ep, const int *episodes, cons
     if (token_ids[r] >= d.vocab) return SPECVLA_ERR_INVALID_ARG;
     if (token_ids[r] < 0 && !embeds) return SPECVLA_ERR_INVALID_ARG;
   }
-  // row table on the host: causal rows, slot = position = index within the episode
-  int *h = ctx->pin_rows;
-  int *h_tok = h, *h_src = h + R, *h_ep = h + 2 * R, *h_pos = h + 3 * R, *h_nvis = h + 4 * R;
-  for (int i = 0; i < n_ep; i++)
-    for (int j = 0; j < lens[i]; j++) {
-      const int r = ea.row0[i] + j;
-      h_tok[r] = token_ids[r];
-      h_src[r] = r;
-      h_ep[r] = episodes[i];
-      h_pos[r] = j;
-      h_nvis[r] = j + 1;
-    }
-  const size_t rb = (size_t)R * sizeof(int);
-  CU(cudaMemcpyAsync(ctx->rt.tok, h_tok, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(ctx->rt.src, h_src, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(ctx->rt.ep, h_ep, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(ctx->rt.pos, h_pos, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(ctx->rt.slot, h_pos, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemcpyAsync(ctx->rt.nvis, h_nvis, rb, cudaMemcpyHostToDevice, st));
-  CU(cudaMemsetAsync(ctx->rt.tbase, 0, rb, st));
-  CU(cudaMemsetAsync(ctx->rt.mask, 0, rb * 4, st));
+  // the token ids go up; the row tables are written on the device
+  memcpy(ctx->pin_rows, token_ids, (size_t)R * sizeof(int));
+  CU(cudaMemcpyAsync(ctx->tok_in, ctx->pin_rows, (size_t)R * sizeof(int), cudaMemcpyHostToDevice, st));
+  LAUNCH(tree::prefill_rows_kernel, dim3((std::max(R, n_ep) + 255) / 256), dim3(256), ea, (const int *)ctx->tok_in,
+         ctx->rt, R, ctx->lm_rows);
 
   const bf16 *emb = static_cast<const bf16 *>(embeds);
   ctx->phase = 1;
   TRY(target_forward(ctx, R, ea, emb, st));
 
   // first token: LM head on each episode's last row
-  int *h_last = h + 5 * R;
-  for (int i = 0; i < n_ep; i++) h_last[i] = ea.aux[i];
-  CU(cudaMemcpyAsync(ctx->lm_rows, h_last, n_ep * sizeof(int), cudaMemcpyHostToDevice, st));
   LAUNCH(epi::gather_rows_kernel, dim3(n_ep), dim3(256), (const bf16 *)ctx->xn.p, ctx->xn.plane,
          (const float *)ctx->ssq, ctx->nt, (const int *)ctx->lm_rows, d.d_model, ctx->lm_in.p, ctx->lm_in.plane,
          ctx->lm_ssq);
@@ -1116,35 +1102,15 @@ static int prefill_enqueue(specvla_ctx *ctx, int n_ep, const int *episodes, cons
   // draft model over the shifted pairs (feature_i, input_{i+1}), i = 0 .. len-2
   if (ctx->has_draft) {
     int Rd = 0;
-    // The draft model's row tables live in their own part of the pinned staging area: the copies
-    // of the target's tables above may still be pending on the stream.
-    int *hd = h + 5 * R + SV_MAX_EP;
-    int *h_tok = hd, *h_src = hd + R, *h_ep = hd + 2 * R, *h_pos = hd + 3 * R, *h_nvis = hd + 4 * R;
-    int *h_fs = hd + 5 * R;                // feature source rows
     EpArgs ed = ea;
     for (int i = 0; i < n_ep; i++) {
       ed.row0[i] = Rd;
       ed.nrows[i] = lens[i] - 1;
-      for (int j = 0; j + 1 < lens[i]; j++) {
-        const int r = Rd++;
-        const int tr = ea.row0[i] + j;     // target row of f_j; the embedding comes from row tr+1
-        h_tok[r] = token_ids[tr + 1];
-        h_src[r] = tr + 1;
-        h_ep[r] = episodes[i];
-        h_pos[r] = j;
-        h_nvis[r] = j + 1;
-        h_fs[r] = tr;
-      }
+      Rd += lens[i] - 1;
     }
     if (Rd > 0) {
-      const size_t db = (size_t)Rd * sizeof(int);
-      CU(cudaMemcpyAsync(ctx->rt.tok, h_tok, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->rt.src, h_src, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->rt.ep, h_ep, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->rt.pos, h_pos, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->rt.slot, h_pos, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->rt.nvis, h_nvis, db, cudaMemcpyHostToDevice, st));
-      CU(cudaMemcpyAsync(ctx->feat_src, h_fs, db, cudaMemcpyHostToDevice, st));
+      LAUNCH(tree::prefill_draft_rows_kernel, dim3((Rd + 255) / 256), dim3(256), ea, (const int *)ctx->tok_in, ctx->rt,
+             Rd, ctx->feat_src);
       LAUNCH(tree::draft_input_kernel, dim3(Rd), dim3(256), ctx->rt, (const int *)ctx->feat_src,
              (const float *)ctx->feat, (const float *)nullptr, 0, (const float *)nullptr, 0.f, emb, ctx->embed,
              d.d_model, ctx->xin.p, ctx->xin.plane);
@@ -1531,10 +1497,10 @@ static int generate_on_device(specvla_ctx *ctx, int n_ep, const int *episodes, c
   CU(cudaGraphLaunch(ctx->loop_exec, st));
   CU(cudaEventRecord(ctx->ev[2], st));
   ChunkState *h = ctx->pin_chunk;
-  EpState *hs = reinterpret_cast<EpState *>(h + 1);
-  CU(cudaMemcpyAsync(h, ctx->chunk, sizeof(ChunkState), cudaMemcpyDeviceToHost, st));
-  CU(cudaMemcpyAsync(hs, ctx->st, sizeof(EpState) * ctx->desc.max_episodes, cudaMemcpyDeviceToHost, st));
-  CU(cudaMemcpyAsync(ctx->pin_small + 4000, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  auto read_back = [&](const void *dev) { return reinterpret_cast<char *>(h) + (static_cast<const char *>(dev) - reinterpret_cast<const char *>(ctx->chunk)); };
+  const EpState *hs = reinterpret_cast<const EpState *>(read_back(ctx->st));
+  const int *h_err = reinterpret_cast<const int *>(read_back(ctx->err));
+  CU(cudaMemcpyAsync(h, ctx->chunk, ctx->chunk_span, cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   ctx->launches += ctx->loop_launches_once + (long long)h->iterations * ctx->loop_launches_iter;
   ctx->feat_valid = false;
@@ -1546,7 +1512,7 @@ static int generate_on_device(specvla_ctx *ctx, int n_ep, const int *episodes, c
     ctx->hTreeRows[e] = 0;
     complete &= h->count[i] >= n_tokens;
   }
-  if (ctx->pin_small[4000] != 0) {
+  if (*h_err != 0) {
     for (int i = 0; i < n_ep; i++) ctx->hP[episodes[i]] = -1;
     return SPECVLA_ERR_TIMEOUT;
   }
