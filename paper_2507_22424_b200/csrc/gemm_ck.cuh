@@ -159,6 +159,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint32_t idesc = instr_desc(2 * tn);
 
   const int npre = n_units < STAGES ? n_units : STAGES;
+  const bool direct = MODE == EPI_SWIGLU && !Q8 && S == 1;   // finished from TMEM, without the partial tile
   const uint64_t pol_w = policy_evict_first();
   // test hook: the K block that is never loaded (-1: none)
   const int withheld = ea.withhold_unit - 1;
@@ -421,6 +422,45 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
     const uint32_t tadr = tmem_base + ((uint32_t)(q * 32) << 16);
     const int col = q * 32 + lane;                       // column within a 128-column half
+    if (direct && have) {
+      // A thread has gate and up of its column in the same TMEM lane, so an unsplit tile is finished
+      // from registers. Two neighbouring lanes exchange a value each per pair of rows, so that both
+      // store two columns of one row. (Prefill of 16 x 296 rows 112.6 -> 111.7 ms, of 290 rows 8.46 ->
+      // 8.37 ms; short tiles measure the same either way.)
+      const int n = tile * 128 + col;
+#pragma unroll 1
+      for (int c0 = 16 * wp; c0 < T; c0 += 32) {
+        uint32_t gh[16], gl[16], uh[16], ul[16];
+        tc_ld16(tadr + c0, gh);
+        tc_ld16(tadr + tn + c0, gl);
+        tc_ld16(tadr + AW + c0, uh);
+        tc_ld16(tadr + AW + tn + c0, ul);
+        tc_wait_ld();
+        float h[16];
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+          const float sc = s_scale[c0 + j < T ? c0 + j : 0];
+          const float g = sc * (__uint_as_float(gh[j]) + __uint_as_float(gl[j]));
+          const float u = sc * (__uint_as_float(uh[j]) + __uint_as_float(ul[j]));
+          h[j] = __fdividef(g, 1.f + __expf(-g)) * u;
+        }
+        const bool odd = lane & 1;
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) {
+          const float got = __shfl_xor_sync(0xffffffffu, odd ? h[j] : h[j + 1], 1);
+          const float v0 = odd ? got : h[j], v1 = odd ? h[j + 1] : got;
+          const int t = c0 + j + (odd ? 1 : 0);
+          const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
+          const float2 hf = __bfloat1622float2(hi);
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
+          if (t < T && n < ea.N) {
+            bf16 *dst = ea.hid + (size_t)(row0 + t) * ea.N + (n & ~1);
+            *reinterpret_cast<__nv_bfloat162 *>(dst) = hi;
+            *reinterpret_cast<__nv_bfloat162 *>(dst + ea.hid_plane) = lo;
+          }
+        }
+      }
+    } else
 #pragma unroll 1
     for (int c0 = 16 * wp; c0 < tn; c0 += 32) {
 #pragma unroll 1
@@ -467,7 +507,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   }
 
-  if (warp >= 2 && warp < 10) {
+  if (warp >= 2 && warp < 10 && !direct) {
     // ------------------------------------------------------------------ epilogue, part 2:
     // rows rank, rank + S, ... of the tile. A thread owns four consecutive columns and every
     // RG-th of those rows (64 column groups x 4 row groups; SwiGLU, whose 128 outputs come
