@@ -911,7 +911,7 @@ inline RowPlan plan_rows(int R, int tiles, int KB, const ClusterFit &fit, bool q
 // ea.tn_chunk; tmXtail: the map for the last chunk (box rows ea.tn_tail).
 inline cudaError_t launch(const CUtensorMap &tmW, const CUtensorMap &tmX, const CUtensorMap &tmXtail,
                           const EpiArgs &ea, int tiles, int KB, int S, int *err, cudaStream_t st, bool pdl) {
-  // (launches of several chunks always take the 128-row instantiation: it alone reads the widths from ea)
+  // (launches of several chunks always take the 128-row instantiation: it alone reads its chunk length from ea)
   switch (ea.T > MAX_T ? MAX_T : tn_of(ea.T)) {
     case 16: return launch_tn<16>(tmW, tmX, tmX, ea, tiles, KB, S, err, st, pdl);
     case 32: return launch_tn<32>(tmW, tmX, tmX, ea, tiles, KB, S, err, st, pdl);

@@ -249,8 +249,8 @@ struct EpiArgs {
   int row0;              // first row of this launch within the call's row range
   int T;                 // rows of this launch; the CTAs of chunk c take rows [chunk_rows c, chunk_rows (c + 1))
   int chunk_rows;        // rows per chunk (<= 128); launches of up to 128 rows are one chunk
-  int tn_chunk, tn_tail; // X box rows = half the MMA width (multiples of 8) of the 128-row instantiation: of
-                         // every chunk but the last, and of the last
+  int tn_chunk, tn_tail; // X box rows = half the MMA width (multiples of 8) of the 64- and 128-row
+                         // instantiations: of every chunk but the last, and of the last
   int raster;            // row chunks whose CTAs run side by side (launches of several chunks)
   int N;                 // output columns (EPI_SWIGLU: F, the width of gate and of up)
   int up_off;            // EPI_SWIGLU: row of W where the up projection starts (F)

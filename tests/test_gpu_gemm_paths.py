@@ -24,3 +24,22 @@ def _check(T, N, K, packed):
 @pytest.mark.parametrize("packed", [True, False])
 def test_many_row_chunks(T, N, K, packed):
     _check(T, N, K, packed)
+
+
+# MMA widths of the 64-row instantiation: the next multiple of eight rows, first and last row of each
+@pytest.mark.parametrize("T", [33, 40, 41, 57, 64, 65])
+def test_widths_between_33_and_64_rows(T):
+    _check(T, 1000, 520, True)
+
+
+def test_operand_off_a_16_byte_boundary():
+    """The split takes X four values at a time only where it starts on 16 bytes."""
+    from paper_2507_22424_b200.binding import gemm
+    T, N, K = 19, 256, 264
+    x = rng.normal(22, 1, (T, K), 1.0, dtype=torch.float32)
+    w = rng.normal_bf16(22, 2, (N, K), 0.02).cuda()
+    buf = torch.empty(T * K + 1, dtype=torch.float32, device="cuda")
+    off = buf[1:].view(T, K)
+    off.copy_(x)
+    assert off.data_ptr() % 16 == 4
+    assert torch.equal(gemm(off, w), gemm(x.cuda(), w))
