@@ -848,7 +848,10 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   ctx->use_l2_prefetch = true;
   ctx->fit = gemm_ck::query_cluster_fit();
   size_t packed_used = 0, q8_used = 0, scale_used = 0;
-  bool pack_ok = true;
+  bool pack_ok = true, cuda_ok = true;
+  // (a failed call here is this call's error and stays with it)
+  auto check = [&](cudaError_t e) { cuda_ok &= e == cudaSuccess; };
+  cudaGetLastError();
   const bool quantise = desc->weight_bits == 8;
   // swiglu: the matrix is [gate; up] stacked ([2F, K]) and is packed as tiles of 128 + 128 rows.
   // q8: a matrix of the quantised target: row scales and int8 codes instead of the bf16 copy.
@@ -874,6 +877,7 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
       q8_used += bytes;
       gemm_tc::row_scale_q8_kernel<<<(N + 7) / 8, 256>>>(w.p, N, K, sc);
       gemm_tc::pack_weights_q8_kernel<<<148 * 8, 256>>>(w.p, N, K, tiles, KB, swiglu ? 1 : 0, F, sc, dst);
+      check(cudaGetLastError());
       w.q8 = dst;
       w.scale = sc;
       return w;
@@ -890,6 +894,7 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
       packed_used += elems;
       gemm_tc::pack_weights_kernel<<<148 * 8, 256>>>(w.p, N, K, tiles, (K + gemm_tc::BK - 1) / gemm_tc::BK,
                                                      swiglu ? 1 : 0, F, dst);
+      check(cudaGetLastError());
       w.packed = dst;
     }
     return w;
@@ -957,7 +962,7 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   ctx->loop_graph = nullptr;
   ctx->loop_exec = nullptr;
   ctx->loop_launches_once = ctx->loop_launches_iter = 0;
-  for (int i = 0; i < 4; i++) cudaEventCreate(&ctx->ev[i]);
+  for (int i = 0; i < 4; i++) check(cudaEventCreate(&ctx->ev[i]));
   ctx->prof_mask = 0;
   ctx->phase = 0;
   ctx->prof_used = 0;
@@ -965,15 +970,20 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   // device-side initialisation: RoPE table, zeroed state
   const int half = desc->head_dim / 2, n = desc->max_seq * half;
   epi::rope_table_kernel<<<(n + 255) / 256, 256>>>(ctx->rope_tab, desc->max_seq, half, (double)desc->rope_theta);
-  cudaMemsetAsync(ctx->st, 0, sizeof(EpState) * desc->max_episodes);
-  cudaMemsetAsync(ctx->trees, 0, sizeof(DevTree) * desc->max_episodes);
-  cudaMemsetAsync(ctx->err, 0, 32 * sizeof(int));
-  auto smem_of = [](auto kernel, int bytes) { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  check(cudaGetLastError());
+  check(cudaMemsetAsync(ctx->st, 0, sizeof(EpState) * desc->max_episodes));
+  check(cudaMemsetAsync(ctx->trees, 0, sizeof(DevTree) * desc->max_episodes));
+  check(cudaMemsetAsync(ctx->err, 0, 32 * sizeof(int)));
+  auto smem_of = [&](auto kernel, int bytes) {
+    check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  };
   smem_of(attn::tree_attention_kernel<128>, attn::smem_bytes<128>());
   smem_of(attn::tree_attention_kernel<64>, attn::smem_bytes<64>());
   smem_of(attn::row_attention_kernel<128>, attn::tc_smem_bytes<128>());
   smem_of(attn::row_attention_kernel<64>, attn::tc_smem_bytes<64>());
-  if (cudaDeviceSynchronize() != cudaSuccess || !pack_ok) {
+  check(cudaDeviceSynchronize());
+  if (!cuda_ok || !pack_ok) {
+    cudaGetLastError();
     cudaFreeHost(ctx->pinned);
     delete ctx;
     return pack_ok ? SPECVLA_ERR_CUDA : SPECVLA_ERR_CAPACITY;
@@ -1792,19 +1802,6 @@ static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, i
   int *err = reinterpret_cast<int *>(base);
   bf16 *limbs = reinterpret_cast<bf16 *>(base + GEMM_HDR);
   const size_t nx = (size_t)T * K;
-  // Two launches: the split (which also clears the status word) starts when the stream's earlier work
-  // is done, the GEMM beside it: its weights do not depend on the split, so the first ring-full of
-  // them lands meanwhile. A call with 512 / 300 / 27 rows of 11008 / 4096 / 11008: 118 / 78 / 62 ->
-  // 109 / 76 / 60 us (the last mostly the host's part).
-  const unsigned blocks = (unsigned)((nx / 4 + epi::THREADS - 1) / epi::THREADS);
-  const int n_status = (int)(GEMM_HDR / sizeof(int));
-  if (reinterpret_cast<uintptr_t>(X) % 16 == 0)
-    epi::split_limbs_kernel<true><<<blocks, epi::THREADS, 0, st>>>(X, nx, limbs, err, n_status);
-  else
-    epi::split_limbs_kernel<false><<<blocks, epi::THREADS, 0, st>>>(X, nx, limbs, err, n_status);
-  if (cudaPeekAtLastError() != cudaSuccess) return SPECVLA_ERR_CUDA;
-  CUtensorMap mw = {}, mx[2];
-  if (W && !gemm_tc::make_w_map(&mw, static_cast<const bf16 *>(W), N, K)) return SPECVLA_ERR_CUDA;
   const int tiles = (N + SV_TILE_ROWS - 1) / SV_TILE_ROWS;
   const int KB = (K + gemm_tc::BK - 1) / gemm_tc::BK;
   gemm_tc::EpiArgs ea = {};
@@ -1817,6 +1814,25 @@ static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, i
   ea.withhold_unit = g_gemm_withhold;
   g_gemm_wait_ns = gemm_tc::WAIT_LIMIT_NS;           // the test hook holds for one call
   g_gemm_withhold = 0;
+  // A launch or a map that is refused fails this call and no other: the error goes with it. (One that
+  // something else left pending is reported once, by the last line, after the work has been enqueued.)
+  auto refused = []() {
+    cudaGetLastError();
+    return SPECVLA_ERR_CUDA;
+  };
+  // Two launches: the split (which also clears the status word) starts when the stream's earlier work
+  // is done, the GEMM beside it: its weights do not depend on the split, so the first ring-full of
+  // them lands meanwhile. A call with 512 / 300 / 27 rows of 11008 / 4096 / 11008: 118 / 78 / 62 ->
+  // 109 / 76 / 60 us (the last mostly the host's part).
+  const unsigned blocks = (unsigned)((nx / 4 + epi::THREADS - 1) / epi::THREADS);
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = launch_cfg(dim3(blocks), dim3(epi::THREADS), st, &at, false);
+  const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
+  if (cudaLaunchKernelEx(&cfg, vec ? epi::split_limbs_kernel<true> : epi::split_limbs_kernel<false>, X, nx, limbs, err,
+                         (int)(GEMM_HDR / sizeof(int))) != cudaSuccess)
+    return refused();
+  CUtensorMap mw = {}, mx[2];
+  if (W && !gemm_tc::make_w_map(&mw, static_cast<const bf16 *>(W), N, K)) return refused();
   const gemm_ck::ClusterFit fit = cluster_fit_of_current_device();
   const gemm_ck::RowPlan plan = gemm_ck::plan_rows(T, tiles, KB, fit, false);
   ea.row0 = 0;
@@ -1827,9 +1843,8 @@ static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, i
   ea.tn_tail = plan.tn_tail;
   if (!gemm_tc::make_x_map(&mx[0], limbs, nx, T, K, plan.tn_chunk) ||
       !gemm_tc::make_x_map(&mx[1], limbs, nx, T, K, plan.tn_tail))
-    return SPECVLA_ERR_CUDA;
-  if (gemm_ck::launch(mw, mx[0], mx[1], ea, tiles, KB, plan.S, err, st, true) != cudaSuccess)
-    return SPECVLA_ERR_CUDA;
+    return refused();
+  if (gemm_ck::launch(mw, mx[0], mx[1], ea, tiles, KB, plan.S, err, st, true) != cudaSuccess) return refused();
   return cudaGetLastError() == cudaSuccess ? SPECVLA_OK : SPECVLA_ERR_CUDA;
 }
 

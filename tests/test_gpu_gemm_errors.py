@@ -1,0 +1,47 @@
+"""A stand-alone product that is refused fails alone: its error and the one-call test hook end with it."""
+import ctypes as C
+
+import pytest
+import torch
+
+from synth_inputs import rng
+
+pytestmark = pytest.mark.gpu
+
+
+def _operands(T, N, K):
+    x = rng.normal(31, 1, (T, K), 1.0, dtype=torch.float32).cuda()
+    w = rng.normal_bf16(31, 2, (N, K), 0.02).cuda()
+    return x, w, x.double() @ w.double().T
+
+
+def _refused_call():
+    """More row chunks than a grid has rows (65535 of 128 rows): the launch is refused on the host."""
+    from paper_2507_22424_b200 import binding as B
+    w = torch.zeros(4, 8, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(B.SpecVLAError) as e:
+        B.gemm(torch.zeros(65536 * 128 + 1, 8, device="cuda"), w)
+    assert e.value.code == -5                                           # SPECVLA_ERR_CUDA
+
+
+@pytest.mark.parametrize("packed", [False, True])
+def test_refused_launch_does_not_fail_later_calls(packed):
+    from paper_2507_22424_b200 import binding as B
+    T, N, K = 19, 512, 264
+    x, w, ref = _operands(T, N, K)
+    p = B.pack_weights(w)
+    _refused_call()
+    for _ in range(3):
+        y = B.gemm_prepacked(x, p, N) if packed else B.gemm(x, w)
+        assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
+
+
+def test_refused_call_takes_the_test_hook_with_it():
+    """The hook holds for the next call, whether that call is launched or refused."""
+    from paper_2507_22424_b200 import binding as B
+    x, w, ref = _operands(16, 256, 512)
+    _refused_call()
+    assert B.lib.specvla_gemm_fault_test(2_000_000, 1) == 0
+    _refused_call()
+    y = B.gemm(x, w)                                                    # an ordinary call: no wait runs out
+    assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (512 ** 0.5) + 1e-6
