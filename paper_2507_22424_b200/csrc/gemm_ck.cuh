@@ -371,6 +371,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       bool ok = wp >= n_units || fetch_codes(wp);
       ok = __all_sync(0xffffffffu, ok);
       for (int it = wp; ok && it < n_units; it += 2) {
+        __syncwarp();                                            // (a vote alone orders no memory)
         if (lane == 0) mbar_arrive(empty_bar(it % STAGES));      // every lane has read its codes
         const int e = it % NE, use = it / NE;
         if (use > 0) ok = mbar_wait(efree_bar(e), (use - 1) & 1, ea.wait_ns);
