@@ -223,11 +223,13 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint32_t rope_off = (uint32_t)(tn * BM * 4);
   float4 xpre0 = make_float4(0.f, 0.f, 0.f, 0.f), xpre1 = xpre0;
 
+  // Every role waits for the preceding kernel before its first bounded wait: a limit covers this
+  // kernel's own work, and an error code is written after what that kernel does to the status word.
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     const uint64_t pol_x = policy_evict_last();
     const bool lead = elect_one();
-    if (!Q8) grid_dep_wait();
+    grid_dep_wait();
     auto load_x = [&](int it, int st) {
       if (it != withheld)
         tma_load_3d(base + st * STAGE + W_STAGE_BYTES, xmap, (kb0 + it) * BK, row0, 0, full_bar(st), pol_x);
@@ -277,6 +279,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     const bool lead = elect_one();
+    grid_dep_wait();
     for (int it = 0, st = 0, ph = 0, e = 0, eph = 0; it < n_units; it++) {
       const bool ok = Q8 ? mbar_wait(xfull_bar(e), eph, ea.wait_ns) && mbar_wait(conv_bar(e), eph, ea.wait_ns)
                          : mbar_wait(full_bar(st), ph, ea.wait_ns);

@@ -45,3 +45,15 @@ def test_refused_call_takes_the_test_hook_with_it():
     _refused_call()
     y = B.gemm(x, w)                                                    # an ordinary call: no wait runs out
     assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (512 ** 0.5) + 1e-6
+
+
+@pytest.mark.parametrize("T,N,K", [(1, 256, 8192), (512, 1024, 4096), (40000, 256, 512)])
+def test_a_wait_limit_covers_the_product_alone(T, N, K):
+    """A limit of 0.2 ms, far above any wait of the product itself, never runs out, however much the
+    operand split in front of it has to do; the status word says so."""
+    from paper_2507_22424_b200 import binding as B
+    x, w, ref = _operands(T, N, K)
+    for _ in range(5):
+        assert B.lib.specvla_gemm_fault_test(200_000, -1) == 0          # no K block is withheld
+        y = B.gemm(x, w)                                                # (raises on a timeout)
+    assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
