@@ -107,6 +107,10 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// Index of "nothing found" in a search for the largest value: every comparison with a NaN is false.
+// Tokens are used as row numbers of the embedding, so a row of NaN logits must still give one.
+constexpr int NO_INDEX = 0x7fffffff;
+__device__ __forceinline__ int found_or(int i, int fallback) { return i == NO_INDEX ? fallback : i; }
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

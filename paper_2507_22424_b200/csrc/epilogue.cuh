@@ -131,15 +131,15 @@ using sv::top2_warp;
 // Greedy token per row from the candidates a GEMM epilogue left: cand[row][0..nc) holds the top-2
 // of each 128-column group of the row's logits (value, column as int bits, second value). One
 // warp per row; ties go to the lowest id; margin = top-1 minus top-2. Column c is token tok_offset + c
-// (the GEMM may have covered only a slice of the vocabulary).
+// (the GEMM may have covered only a slice of the vocabulary). A row of NaN gets column lo, margin NaN.
 __global__ void __launch_bounds__(128)
-argmax_merge_kernel(const float4 *__restrict__ cand, int nc, int rows, int tok_offset, int *__restrict__ greedy,
-                    float *__restrict__ margin) {
+argmax_merge_kernel(const float4 *__restrict__ cand, int nc, int rows, int lo, int tok_offset,
+                    int *__restrict__ greedy, float *__restrict__ margin) {
   pdl_launch();
   pdl_wait();
   const int t = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= rows) return;
-  Top2 best{-INFINITY, -INFINITY, 0x7fffffff};
+  Top2 best{-INFINITY, -INFINITY, NO_INDEX};
   for (int i = lane; i < nc; i += 32) {
     const float4 c = cand[(size_t)t * nc + i];
     const Top2 other{c.x, c.z, __float_as_int(c.y)};
@@ -147,7 +147,7 @@ argmax_merge_kernel(const float4 *__restrict__ cand, int nc, int rows, int tok_o
   }
   top2_warp(best);
   if (lane == 0) {
-    greedy[t] = best.i1 + tok_offset;
+    greedy[t] = found_or(best.i1, lo) + tok_offset;
     margin[t] = best.v1 - best.v2;
   }
 }
@@ -179,7 +179,7 @@ logsoftmax_topk_kernel(const float *__restrict__ logits, int V, int lo, int hi, 
   const float lse = mx + logf(se);
   for (int k = 0; k < SV_TOPK; k++) {
     float bv = -INFINITY;
-    int bi = 0x7fffffff;
+    int bi = NO_INDEX;
     for (int v = lo + threadIdx.x; v < hi; v += blockDim.x) {
       bool taken = false;
       for (int j = 0; j < k; j++) taken |= (chosen[j] == v);
@@ -198,6 +198,7 @@ logsoftmax_topk_kernel(const float *__restrict__ logits, int V, int lo, int hi, 
     if (threadIdx.x == 0) {
       for (int w = 1; w < THREADS / 32; w++)
         if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
+      bi = found_or(bi, min(lo + k, hi - 1));
       chosen[k] = bi;
       top_tok[t * SV_TOPK + k] = bi + tok_offset;
       top_lp[t * SV_TOPK + k] = bv - lse;

@@ -592,7 +592,7 @@ __device__ __forceinline__ void finish_phase(const Params &p, const Op &o, const
         float *outp = o.post == POST_ARGMAX ? p.logits_out : o.out;
         if (outp && n < o.N) *reinterpret_cast<float4 *>(outp + (size_t)t * o.ldo + n) = ov;
         if (o.post == POST_ARGMAX) {
-          epi::Top2 bb{-INFINITY, -INFINITY, 0x7fffffff};
+          epi::Top2 bb{-INFINITY, -INFINITY, NO_INDEX};
           const float vv[4] = {ov.x, ov.y, ov.z, ov.w};
 #pragma unroll
           for (int e2 = 0; e2 < 4; e2++)
@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_pk_kernel(const __grid_con
       if (o.post == POST_ARGMAX) {
         // one warp per row merges the per-128-column candidates (ties to the lowest id)
         for (int t = gw; t < T; t += GW) {
-          epi::Top2 b{-INFINITY, -INFINITY, 0x7fffffff};
+          epi::Top2 b{-INFINITY, -INFINITY, NO_INDEX};
           for (int i = lane; i < 2 * o.tiles; i += 32) {
             const float4 cd = __ldcg(p.cand + (size_t)t * (2 * o.tiles) + i);
             epi::Top2 other{cd.x, cd.z, __float_as_int(cd.y)};
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_pk_kernel(const __grid_con
           }
           top2_warp(b);
           if (lane == 0) {
-            p.greedy[t] = b.i1;
+            p.greedy[t] = found_or(b.i1, o.lo);
             p.margin[t] = b.v1 - b.v2;
           }
         }
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_pk_kernel(const __grid_con
           int chosen[SV_TOPK];
           for (int k = 0; k < SV_TOPK; k++) {
             float bv = -INFINITY;
-            int bi = 0x7fffffff;
+            int bi = NO_INDEX;
             for (int v = o.lo + lane; v < o.hi; v += 32) {
               bool taken = false;
               for (int jj = 0; jj < k; jj++) taken |= (chosen[jj] == v);
@@ -967,6 +967,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_pk_kernel(const __grid_con
               const int oi2 = __shfl_xor_sync(0xffffffffu, bi, of);
               if (ov > bv || (ov == bv && oi2 < bi)) { bv = ov; bi = oi2; }
             }
+            bi = found_or(bi, min(o.lo + k, o.hi - 1));
             chosen[k] = bi;
             if (lane == 0) {
               p.top_tok[t * SV_TOPK + k] = bi + o.tok_offset;

@@ -620,7 +620,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           if (ea.out && col_ok) *reinterpret_cast<float4 *>(ea.out + row * ea.ldo + n) = ov;
           if (ea.cand) {
             // greedy argmax, first step: the top-2 of this warp's 128 columns over [lo, hi)
-            sv::Top2 b{-INFINITY, -INFINITY, 0x7fffffff};
+            sv::Top2 b{-INFINITY, -INFINITY, NO_INDEX};
             const float vv[4] = {ov.x, ov.y, ov.z, ov.w};
   #pragma unroll
             for (int e = 0; e < 4; e++)
@@ -659,7 +659,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           unsigned taken = 0;
           for (int k = 0; k < SV_TOPK; k++) {
             float bv = -INFINITY;
-            int bi = 0x7fffffff;
+            int bi = NO_INDEX;
   #pragma unroll
             for (int e = 0; e < 4; e++)
               if (in[e] && !((taken >> e) & 1u) && (xv[e] > bv || (xv[e] == bv && n + e < bi))) {
@@ -684,7 +684,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             const int i0 = s_xi[rg][0], i1 = s_xi[rg][1];
             const bool first = v0 > v1 || (v0 == v1 && i0 < i1);
             bv = first ? v0 : v1;
-            bi = first ? i0 : i1;
+            bi = found_or(first ? i0 : i1, min(ea.lo + k, min(ea.hi, ea.N) - 1));
             pair_sync();
             if (bi >= n && bi < n + 4) taken |= 1u << (bi - n);
             if ((et & 63) == 0) {

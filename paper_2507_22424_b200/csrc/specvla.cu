@@ -598,7 +598,7 @@ int lm_head_greedy(specvla_ctx *ctx, const XBuf &A, const float *ssq, int rows, 
   TRY(gemm(ctx, A, W, rows, e, st, SPECVLA_PROF_LM_HEAD));
   const int nc = 2 * ((W.N + SV_TILE_ROWS - 1) / SV_TILE_ROWS);
   LAUNCH(epi::argmax_merge_kernel, dim3((rows + 3) / 4), dim3(128), (const float4 *)ctx->cand, nc, rows,
-         act_rows ? d.action_base : 0, ctx->greedy, ctx->margin);
+         e.lo, act_rows ? d.action_base : 0, ctx->greedy, ctx->margin);
   return SPECVLA_OK;
 }
 

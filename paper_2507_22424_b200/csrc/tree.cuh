@@ -283,7 +283,8 @@ grow_input_kernel(EpArgs a, int level, int branch, int expand_next, const int *_
   if (k < m) {
     const int j = k / branch, b = k - j * branch;
     const int p = s_sel_old[j], srow = a.row0[i] + j, n = begin + k;
-    const float sc = tr.score[p] + top_lp[srow * SV_TOPK + b];
+    float sc = tr.score[p] + top_lp[srow * SV_TOPK + b];
+    if (!(sc == sc)) sc = -INFINITY;                // ranks below need an order: NaN compares with nothing
     tr.tok[n] = top_tok[srow * SV_TOPK + b];
     tr.parent[n] = p;
     tr.depth[n] = level + 1;
