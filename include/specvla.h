@@ -167,8 +167,10 @@ int specvla_destroy(specvla_ctx *ctx);
  *       stream serialisation (a GEMM streams weights while its predecessor drains).
  *   SPECVLA_OPT_L2_PREFETCH         1: a GEMM of the per-GEMM path prefetches the head of the next
  *       matrix into L2.
- *   SPECVLA_OPT_WAIT_LIMIT_NS       limit of every device-side wait of the persistent kernel in
- *       nanoseconds (default 2e9); a wait that runs out makes the call return SPECVLA_ERR_TIMEOUT.
+ *   SPECVLA_OPT_WAIT_LIMIT_NS       limit of every device-side wait of the context's kernels (GEMMs,
+ *       attention, the persistent forward) in nanoseconds (default 2e9). A wait that runs out makes the
+ *       call that reads results back return SPECVLA_ERR_TIMEOUT, once; the context stays usable, the
+ *       episodes of that call have to be prefilled again (those of specvla_score_tree have not).
  *   SPECVLA_OPT_DEVICE_LOOP         1 (default): specvla_generate_action runs the iterations of
  *       Algorithm 1 as ONE launch of a CUDA graph whose while node repeats draft tree, verification
  *       and the appending of the emitted tokens until the chunk is complete; the host reads tokens,
@@ -177,12 +179,18 @@ int specvla_destroy(specvla_ctx *ctx);
  *       prefix + n_tokens + depth + tree rows; otherwise, with 0, and when the driver refuses the
  *       graph (remembered until this option is set again), the host runs the loop and reads the
  *       accepted length back every iteration. Same tokens either way; specvla_stats.device_loop
- *       says which loop ran. */
+ *       says which loop ran.
+ *   SPECVLA_OPT_WITHHOLD_GEMM, SPECVLA_OPT_WITHHOLD_KEYS  failure-handling test hooks, each good for one
+ *       launch: every CTA of the next GEMM withholds the K block of that index within its K range / of
+ *       the next attention launch with more than 96 (32-row block, head) pairs the key tile (64 slots)
+ *       of that index, so that the waits for it run out (set a limit). -1: none. */
 #define SPECVLA_OPT_PERSISTENT_FORWARD 1
 #define SPECVLA_OPT_DEPENDENT_LAUNCH   2
 #define SPECVLA_OPT_L2_PREFETCH        3
 #define SPECVLA_OPT_WAIT_LIMIT_NS      4
 #define SPECVLA_OPT_DEVICE_LOOP        5
+#define SPECVLA_OPT_WITHHOLD_GEMM      6
+#define SPECVLA_OPT_WITHHOLD_KEYS      7
 int specvla_set_option(specvla_ctx *ctx, int option, long long value);
 
 /* Forgets an episode's state (its caches are simply overwritten by the next prefill). */

@@ -16,6 +16,7 @@ MAX_DEPTH = 8
 MAX_TREE_ROWS = 128
 
 OPT_PERSISTENT_FORWARD, OPT_DEPENDENT_LAUNCH, OPT_L2_PREFETCH, OPT_WAIT_LIMIT_NS, OPT_DEVICE_LOOP = 1, 2, 3, 4, 5
+OPT_WITHHOLD_GEMM, OPT_WITHHOLD_KEYS = 6, 7
 BUF_GREEDY, BUF_MARGIN, BUF_FEATURES, BUF_PATH, BUF_STATE, BUF_TOPK_TOK, BUF_TOPK_LP = 1, 2, 3, 4, 5, 6, 7
 
 

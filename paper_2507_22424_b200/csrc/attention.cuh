@@ -49,6 +49,7 @@ struct Args {
   int splits;              // few-row launches: key slices per row block; the cluster is (splits, 1, 1)
   unsigned long long wait_ns;   // long launches: limit of every mbarrier wait, and the status word
   int *err;
+  int withhold_tile;       // test hook (SPECVLA_OPT_WITHHOLD_KEYS), long launches: key tile never reported (-1: none)
 };
 
 __host__ __device__ inline int blocks_of(const EpArgs &ea, int rows) {
@@ -636,7 +637,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(k_full(b));
+      if (lane == 0 && t != a.withhold_tile) mbar_arrive(k_full(b));
       if (t + 1 < tiles) load_k(t + 1);
       ok = t < 2 || mbar_wait(v_free(b), ((t >> 1) - 1) & 1, a.wait_ns);
       if (!__all_sync(0xffffffffu, ok)) {

@@ -255,7 +255,7 @@ struct EpiArgs {
   int N;                 // output columns (EPI_SWIGLU: F, the width of gate and of up)
   int up_off;            // EPI_SWIGLU: row of W where the up projection starts (F)
   unsigned long long wait_ns;   // limit of every mbarrier wait
-  int withhold_unit;     // test hook (specvla_gemm_fault_test): > 0: the producer of every CTA skips its
+  int withhold_unit;     // test hook (specvla_gemm_fault_test, SPECVLA_OPT_WITHHOLD_GEMM): > 0: the producer of every CTA skips its
                          // (withhold_unit - 1)-th K block, so the waits for it run out; 0: off
   const signed char *wq8;   // int8 codes of the weights in the same unit order (16 KB per unit, see
                             // pack_weights_q8_kernel), or NULL; wscale[n] = scale of weight row n

@@ -8,8 +8,10 @@
 #include <string.h>
 
 #include <algorithm>
+#include <climits>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "attention.cuh"
@@ -117,6 +119,8 @@ struct specvla_ctx {
   bf16 *pk_xn, *pk_ao, *pk_hid;
   unsigned *pk_bar;
   unsigned long long wait_ns;   // limit of every device-side wait
+  int withhold_gemm, withhold_keys;   // test hooks: 1 + K block / key tile withheld by the next launch (0: none)
+  bool capturing;               // launches are being recorded (the test hooks are for launches that run)
   const float *last_ssq;        // sums of squares (and their slots per row) left by the last target forward
   int last_nt;
 
@@ -385,6 +389,7 @@ int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs
   ea.wq8 = W.q8;
   ea.wscale = W.scale;
   ea.wait_ns = ctx->wait_ns;
+  if (!ctx->capturing) ea.withhold_unit = std::exchange(ctx->withhold_gemm, 0);
   ea.inv_k = 1.f / (float)W.K;
   ea.eps = ctx->desc.rms_eps;
   const bool prof = (ctx->prof_mask & ctx->phase) && 2 * (ctx->prof_used + 1) <= (int)ctx->prof_ev.size();
@@ -470,6 +475,7 @@ int attention(specvla_ctx *ctx, const EpArgs &rows, const float *cache, size_t e
   a.out_plane = ctx->ao.plane;
   a.wait_ns = ctx->wait_ns;
   a.err = ctx->err;
+  a.withhold_tile = -1;
   const int blocks = attn::blocks_of(rows, attn::RB);
   if (blocks < 1) return SPECVLA_OK;
   const int ctas = blocks * d.n_heads;
@@ -487,6 +493,7 @@ int attention(specvla_ctx *ctx, const EpArgs &rows, const float *cache, size_t e
     CU(d.head_dim == 128 ? cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<128>, rows, a)
                          : cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<64>, rows, a));
   } else {
+    if (!ctx->capturing) a.withhold_tile = std::exchange(ctx->withhold_keys, 0) - 1;
     cudaLaunchConfig_t cfg = launch_cfg(dim3(d.n_heads, attn::blocks_of(rows, attn::TC_ROWS)), dim3(attn::TC_THREADS), st,
                                         &at[0], ctx->use_pdl);
     cfg.dynamicSmemBytes = d.head_dim == 128 ? attn::tc_smem_bytes<128>() : attn::tc_smem_bytes<64>();
@@ -931,6 +938,8 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
                          wmat(dw->wd, D, F), dw->norm1, dw->norm2};
   }
   ctx->wait_ns = 2000000000ull;
+  ctx->withhold_gemm = ctx->withhold_keys = 0;
+  ctx->capturing = false;
   ctx->last_ssq = ctx->ssq;
   ctx->last_nt = ctx->nt;
   ctx->pk_ok = false;
@@ -1028,6 +1037,11 @@ int specvla_set_option(specvla_ctx *ctx, int option, long long value) {
       if (value < 1000) return SPECVLA_ERR_INVALID_ARG;
       ctx->wait_ns = (unsigned long long)value;
       break;
+    case SPECVLA_OPT_WITHHOLD_GEMM:
+    case SPECVLA_OPT_WITHHOLD_KEYS:
+      if (value < -1 || value > INT_MAX - 1) return SPECVLA_ERR_INVALID_ARG;
+      (option == SPECVLA_OPT_WITHHOLD_GEMM ? ctx->withhold_gemm : ctx->withhold_keys) = (int)value + 1;
+      break;
     default: return SPECVLA_ERR_INVALID_ARG;
   }
   return SPECVLA_OK;
@@ -1043,6 +1057,15 @@ int specvla_reset(specvla_ctx *ctx, int episode) {
 static int prefill_enqueue(specvla_ctx *ctx, int n_ep, const int *episodes, const void *embeds,
                            const int *token_ids, const int *lens, float *logits_out, cudaStream_t st);
 
+// A device-side wait of the call gave up. Said once: the status word is cleared, so that the next call
+// answers for itself. The episodes listed have lost their state and must be prefilled again.
+static int timed_out(specvla_ctx *ctx, int n_ep, const int *episodes, cudaStream_t st) {
+  for (int i = 0; i < n_ep; i++) ctx->hP[episodes[i]] = -1;
+  CU(cudaMemsetAsync(ctx->err, 0, sizeof(int), st));
+  CU(cudaStreamSynchronize(st));
+  return SPECVLA_ERR_TIMEOUT;
+}
+
 int specvla_prefill(specvla_ctx *ctx, int n_ep, const int *episodes, const void *embeds,
                     const int *token_ids, const int *lens, int *first_token_out, float *logits_out,
                     void *stream) {
@@ -1053,10 +1076,7 @@ int specvla_prefill(specvla_ctx *ctx, int n_ep, const int *episodes, const void 
   CU(cudaMemcpyAsync(h_g + 4000, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   prof_collect(ctx);
-  if (h_g[4000] != 0) {
-    for (int i = 0; i < n_ep; i++) ctx->hP[episodes[i]] = -1;
-    return SPECVLA_ERR_TIMEOUT;
-  }
+  if (h_g[4000] != 0) return timed_out(ctx, n_ep, episodes, st);
   for (int i = 0; i < n_ep; i++)
     if (first_token_out) first_token_out[i] = h_g[i];
   return SPECVLA_OK;
@@ -1293,7 +1313,7 @@ static int finish_verify(specvla_ctx *ctx, const EpArgs &ea, int *accept_len_out
   CU(cudaMemcpyAsync(h + 4000, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   prof_collect(ctx);
-  if (h[4000] != 0) return SPECVLA_ERR_TIMEOUT;
+  if (h[4000] != 0) return timed_out(ctx, n_ep, ea.eps, st);
   for (int i = 0; i < n_ep; i++) {
     const int e = ea.eps[i], m = h[i];
     if (m < 0 || m > SV_MAX_DEPTH) return SPECVLA_ERR_BAD_STATE;
@@ -1391,7 +1411,7 @@ int specvla_score_tree(specvla_ctx *ctx, int n_ep, const int *episodes, const sp
   CU(cudaMemcpyAsync(h + 4000, ctx->err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   prof_collect(ctx);
-  if (h[4000] != 0) return SPECVLA_ERR_TIMEOUT;
+  if (h[4000] != 0) return timed_out(ctx, 0, nullptr, st);          // (no episode's state has changed)
   for (int k = 0; k < R; k++) greedy_out[k] = h[k];
   return SPECVLA_OK;
 }
@@ -1457,7 +1477,9 @@ static int build_loop_graph(specvla_ctx *ctx, int n_ep, const int *episodes, con
            (const int *)ctx->out_tok, (const int *)ctx->err, handle);
     return SPECVLA_OK;
   };
+  ctx->capturing = true;
   const int rc = record();
+  ctx->capturing = false;
   cudaGraph_t captured = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(st, &captured);
   ctx->loop_launches_iter = ctx->launches - before;
@@ -1522,10 +1544,7 @@ static int generate_on_device(specvla_ctx *ctx, int n_ep, const int *episodes, c
     ctx->hTreeRows[e] = 0;
     complete &= h->count[i] >= n_tokens;
   }
-  if (*h_err != 0) {
-    for (int i = 0; i < n_ep; i++) ctx->hP[episodes[i]] = -1;
-    return SPECVLA_ERR_TIMEOUT;
-  }
+  if (*h_err != 0) return timed_out(ctx, n_ep, episodes, st);
   if (!complete) return SPECVLA_ERR_BAD_STATE;
   for (int i = 0; i < n_ep; i++)
     for (int k = 0; k < n_tokens; k++) tokens_out[(size_t)i * n_tokens + k] = h->tokens[i][k];
