@@ -483,15 +483,18 @@ int attention(specvla_ctx *ctx, const EpArgs &rows, const float *cache, size_t e
   if (ctas <= attn::FEW_CTAS) {
     // the slices of a row block are one cluster (they merge through distributed shared memory)
     a.splits = std::max(1, std::min(attn::MAX_SPLIT_CTAS / ctas, attn::MAX_SPLITS));
-    cudaLaunchConfig_t cfg = launch_cfg(dim3(blocks * a.splits, d.n_heads), dim3(attn::THREADS), st, &at[0], ctx->use_pdl);
+    const bool sliced = a.splits > 1;
+    cudaLaunchConfig_t cfg = launch_cfg(sliced ? dim3(blocks * a.splits, d.n_heads) : dim3(d.n_heads, blocks),
+                                        dim3(attn::THREADS), st, &at[0], ctx->use_pdl);
     at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
     at[cfg.numAttrs].val.clusterDim.x = a.splits;
     at[cfg.numAttrs].val.clusterDim.y = 1;
     at[cfg.numAttrs].val.clusterDim.z = 1;
     cfg.numAttrs++;
     cfg.dynamicSmemBytes = d.head_dim == 128 ? attn::smem_bytes<128>() : attn::smem_bytes<64>();
-    CU(d.head_dim == 128 ? cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<128>, rows, a)
-                         : cudaLaunchKernelEx(&cfg, attn::tree_attention_kernel<64>, rows, a));
+    CU(cudaLaunchKernelEx(&cfg, d.head_dim == 128 ? (sliced ? attn::tree_attention_kernel<128, true> : attn::tree_attention_kernel<128, false>)
+                                                  : (sliced ? attn::tree_attention_kernel<64, true> : attn::tree_attention_kernel<64, false>),
+                          rows, a));
   } else {
     if (!ctx->capturing) a.withhold_tile = std::exchange(ctx->withhold_keys, 0) - 1;
     cudaLaunchConfig_t cfg = launch_cfg(dim3(d.n_heads, attn::blocks_of(rows, attn::TC_ROWS)), dim3(attn::TC_THREADS), st,
@@ -986,8 +989,10 @@ int specvla_create(const specvla_model_desc *desc, const specvla_weights *tw,
   auto smem_of = [&](auto kernel, int bytes) {
     check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   };
-  smem_of(attn::tree_attention_kernel<128>, attn::smem_bytes<128>());
-  smem_of(attn::tree_attention_kernel<64>, attn::smem_bytes<64>());
+  smem_of(attn::tree_attention_kernel<128, true>, attn::smem_bytes<128>());
+  smem_of(attn::tree_attention_kernel<128, false>, attn::smem_bytes<128>());
+  smem_of(attn::tree_attention_kernel<64, true>, attn::smem_bytes<64>());
+  smem_of(attn::tree_attention_kernel<64, false>, attn::smem_bytes<64>());
   smem_of(attn::row_attention_kernel<128>, attn::tc_smem_bytes<128>());
   smem_of(attn::row_attention_kernel<64>, attn::tc_smem_bytes<64>());
   check(cudaDeviceSynchronize());

@@ -18,20 +18,20 @@ DESCS = [C.ModelDesc(n_layers=2, d_model=8 * hd, n_heads=8, head_dim=hd, d_ffn=6
          for hd in (64, 128)]
 
 
-@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
-@pytest.mark.parametrize("n_ep", [16, 60])
-def test_batched_rows_equal_single_episodes(desc, n_ep):
+def _batched_equals_single(desc, lens, tree_rows, seed, max_seq=320, oracle_eps=(1, 7)):
+    """Prefill and scoring of all episodes in one call against one call per episode; logits of
+    `oracle_eps` against the oracle."""
     w = data.make_weights(desc, 31)
-    rng = random.Random(n_ep)
-    edges = [65, 31, 97, 64, 33, 128, 96, 129, 63, 127]
-    lens = [edges[i % len(edges)] if n_ep == 60 or i % 2 == 0 else 70 + i for i in range(n_ep)]
+    rng = random.Random(seed)
+    n_ep = len(lens)
     ids = [[rng.randrange(desc.action_base) for _ in range(n)] for n in lens]
-    gpu = G.make_gpu(desc, G.to_cuda(w), max_seq=320, max_episodes=n_ep, max_rows=sum(lens), action_only=True)
+    gpu = G.make_gpu(desc, G.to_cuda(w), max_seq=max_seq, max_episodes=n_ep, max_rows=max(sum(lens), sum(tree_rows)),
+                     action_only=True)
     embeds = torch.zeros(sum(lens), desc.d_model, dtype=torch.bfloat16, device="cuda")
     eps = list(range(n_ep))
     trees = []
     for e in eps:
-        tok, par, dep = data.random_tree([27, 40, 65][e % 3], desc, seed=e, max_depth=8, root_token=None)
+        tok, par, dep = data.random_tree(tree_rows[e], desc, seed=e, max_depth=8, root_token=None)
         trees.append(dict(tokens=[desc.action_base + e] + list(tok)[1:], parent=list(par), depth=list(dep)))
     first, logits = gpu.prefill(eps, embeds, sum(ids, []), lens, want_logits=True)
     greedy = gpu.score_tree(eps, trees)
@@ -50,8 +50,26 @@ def test_batched_rows_equal_single_episodes(desc, n_ep):
         r0 += len(g1)
     assert checked > 0.9 * len(greedy)
     orc = SpecVLAOracle(desc, w)
-    for e in (1, 7):
+    for e in oracle_eps:
         embeds_e, ids_e = torch.zeros(lens[e], desc.d_model, dtype=torch.bfloat16), torch.tensor(ids[e])
         _, ref, _ = orc.prefill(embeds_e, ids_e, want_logits=True)
         assert (logits[e].cpu().double() - ref.reshape(-1)).abs().max() < 1e-3, (e, lens[e])
     gpu.close()
+
+
+@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
+@pytest.mark.parametrize("n_ep", [16, 60])
+def test_batched_rows_equal_single_episodes(desc, n_ep):
+    edges = [65, 31, 97, 64, 33, 128, 96, 129, 63, 127]
+    lens = [edges[i % len(edges)] if n_ep == 60 or i % 2 == 0 else 70 + i for i in range(n_ep)]
+    _batched_equals_single(desc, lens, [[27, 40, 65][e % 3] for e in range(n_ep)], n_ep)
+
+
+# 75 to 96 (row block, head) pairs: the few-row kernel with one slice; a block of one row, a full one and
+# ragged ones, and the first and last count of it
+@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
+@pytest.mark.parametrize("lens", [[32, 1, 31, 17, 5, 32, 29, 2, 32, 16], [64, 33, 31, 62, 1, 32, 64, 32]])
+def test_one_slice_equals_single_episodes(desc, lens):
+    blocks = sum((n + 31) // 32 for n in lens) * desc.n_heads
+    assert 75 <= blocks <= 96, blocks
+    _batched_equals_single(desc, lens, [[32, 27, 1][e % 3] for e in range(len(lens))], 3)
