@@ -448,6 +448,12 @@ tree_attention_kernel(const EpArgs ea, const Args a) {
 //               j DH / 4 + i is dim 4 i + j, and so is column j DH / 4 + i of O;
 //   warp 12     issues the MMAs: S = Q K^T (hi hi in one accumulator, hi lo + lo hi in another, two
 //               buffers), O += P V (three products).
+// A row's weight of a slot that it does not see is zero, and zero times a value that is not finite is
+// NaN: in a block of 128 causal rows one such V row would reach up to 127 rows before it (32 in the
+// few-row kernel, whose tiles 32 rows share). So once the context has cached K and V of a row that is
+// not finite (the QKV GEMM, which has the row's sum of squares, says so in a flag), the loaders write
+// zeros in place of such values, and the rows that do see them get their NaN on the way out. (Checked in
+// every loader, without that flag, it cost 1 us per launch; in the finishing loop of QKV, 0.2 us.)
 // The scores of tile t + 1 are computed while the softmax of tile t runs. Arithmetic as in the few-row
 // kernel: 16 mantissa bits per operand, fp32 accumulation and softmax.
 // Per launch (32 heads of 128; the mma.sync kernel with one CTA per 32 rows before): 16 prefixes of
@@ -501,7 +507,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
   auto kv_base = [&](int b) { return base + (uint32_t)(2 * QB + b * 4 * KVB); };
   __shared__ __align__(8) unsigned long long s_bar[10];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_clean, s_non_finite;
   const uint32_t bars = smem_u32(s_bar);
   auto k_full = [&](int b) { return bars + 8u * b; };           // the loaders have written K (V) of buffer b
   auto v_full = [&](int b) { return bars + 8u * (2 + b); };
@@ -519,7 +525,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
     }
     mbar_init(p_full, 4);
     mbar_init(o_full, 1);
-    s_fail = 0;
+    s_fail = s_non_finite = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 12) {
@@ -540,6 +546,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
   const float *kbase = a.cache + (size_t)ea.eps[ei] * a.ep_stride + (size_t)h * DH;
   const float *vbase = kbase + (size_t)a.max_seq * hd;
 
+  if (tid == TC_THREADS - 1) s_clean = a.err[SV_NON_FINITE_V];
   // last slot that any row sees: every warp finds it for itself
   int kmax = 0;
   {
@@ -635,6 +642,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  const bool clean = s_clean != 0;
   auto fail = [&](int code) {
     atomicExch(a.err, code);
     s_fail = 1;
@@ -666,6 +674,23 @@ row_attention_kernel(const EpArgs ea, const Args a) {
         if (lane == 0) fail(SV_ERR_WAIT_EMPTY);
         break;
       }
+      if (clean) {
+        bool bad = false;
+        auto drop = [&](float &x) {
+          if (!limb_finite(x)) {
+            x = 0.f;
+            bad = true;
+          }
+        };
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          drop(vr[j].x);
+          drop(vr[j].y);
+          drop(vr[j].z);
+          drop(vr[j].w);
+        }
+        if (bad) s_non_finite = 1;
+      }
       if (vg < TC_KEYS / 8) {
         const float v[4][8] = {{vr[0].x, vr[1].x, vr[2].x, vr[3].x, vr[4].x, vr[5].x, vr[6].x, vr[7].x},
                                {vr[0].y, vr[1].y, vr[2].y, vr[3].y, vr[4].y, vr[5].y, vr[6].y, vr[7].y},
@@ -683,6 +708,8 @@ row_attention_kernel(const EpArgs ea, const Args a) {
       if (lane == 0) mbar_arrive(v_full(b));
       if (t + 1 < tiles) load_v(t + 1);
     }
+    __syncwarp();
+    if (clean) asm volatile("bar.arrive 1, %0;" ::"n"(128 + TC_LOADERS) : "memory");   // s_non_finite is final
   } else if (warp == 12) {
     // ------------------------------------------------------------------ MMA issuer
     const bool lead = elect_one();
@@ -870,6 +897,28 @@ row_attention_kernel(const EpArgs ea, const Args a) {
         const size_t idx = (size_t)(row0 + r) * hd + h * DH + c;
         *reinterpret_cast<uint4 *>(a.out + idx) = *reinterpret_cast<const uint4 *>(oh + (i / C8) * LD + c);
         *reinterpret_cast<uint4 *>(a.out + a.out_plane + idx) = *reinterpret_cast<const uint4 *>(ol + (i / C8) * LD + c);
+      }
+    }
+    __syncwarp();
+    if (clean) {
+      asm volatile("bar.sync 1, %0;" ::"n"(128 + TC_LOADERS) : "memory");
+      if (ok && s_non_finite) {
+        // NaN for the rows of this warp that see a slot whose V is not finite, in the dims where it is not
+#pragma unroll 1
+        for (int slot = 0; slot < kmax; slot++) {
+          const int bit = slot - tb;
+          const unsigned long long m64 = bit < 64 ? mlo : mhi;
+          const unsigned sees = __ballot_sync(0xffffffffu, slot < nv || (bit >= 0 && bit < 128 && ((m64 >> (bit & 63)) & 1ull)));
+#pragma unroll 1
+          for (int c = lane; c < DH; c += 32) {
+            if (limb_finite(vbase[(size_t)slot * hd + c])) continue;
+#pragma unroll 1
+            for (unsigned rest = sees; rest; rest &= rest - 1) {
+              const size_t idx = (size_t)(row0 + warp * 32 + __ffs(rest) - 1) * hd + h * DH + c;
+              a.out[idx] = a.out[a.out_plane + idx] = __float2bfloat16(NAN);
+            }
+          }
+        }
       }
     }
     tc_fence_before();

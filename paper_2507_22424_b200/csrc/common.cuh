@@ -102,6 +102,12 @@ __device__ __forceinline__ void store_limbs4(bf16 *hi_plane, size_t plane, size_
   store_bf16x4(hi_plane + plane + idx, make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w));
 }
 
+// Whether a value and its bf16 limb are finite.
+__device__ __forceinline__ bool limb_finite(float v) { return fabsf(v) <= 3.3895314e38f; }
+// Residual rows with a sum of squares up to here are finite, and so are their normalised keys and values,
+// unless the weights make them infinite for every row.
+constexpr float FINITE_ROW_SSQ = 1e30f;
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

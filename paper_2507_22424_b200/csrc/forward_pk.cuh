@@ -871,6 +871,7 @@ __global__ void __launch_bounds__(THREADS, 1) forward_pk_kernel(const __grid_con
           for (int i = lane; i < p.nt; i += 32) ss += __ldcg(p.ssq + t * p.nt + i);
           ss = warp_sum(ss);
           if (lane == 0) s_scale[t] = rsqrtf(ss / (float)p.d + p.eps);
+          if (lane == 0 && !(ss <= FINITE_ROW_SSQ)) p.err[SV_NON_FINITE_V] = 1;
         }
       }
       const int U = o.tiles * o.KB;

@@ -329,6 +329,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         float ss = 0.f;
         for (int j = 0; j < ea.nt_in; j++) ss += ea.ssq_in[(size_t)(row0 + et) * ea.nt_in + j];
         sc = rsqrtf(ss * ea.inv_k + ea.eps);
+        if (MODE == EPI_QKV && !(ss <= FINITE_ROW_SSQ)) err[SV_NON_FINITE_V] = 1;
       }
       s_scale[et] = sc;
       if (MODE == EPI_QKV) {

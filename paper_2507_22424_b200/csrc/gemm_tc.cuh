@@ -225,6 +225,7 @@ __host__ __device__ constexpr uint32_t instr_desc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
+#define SV_NON_FINITE_V 1        // the word after the status word: 1 once keys and values of a row that is not finite were cached
 #define SV_ERR_WAIT_EMPTY 1
 #define SV_ERR_WAIT_FULL 2
 #define SV_ERR_WAIT_TMEM_EMPTY 3

@@ -73,3 +73,41 @@ def test_one_slice_equals_single_episodes(desc, lens):
     blocks = sum((n + 31) // 32 for n in lens) * desc.n_heads
     assert 75 <= blocks <= 96, blocks
     _batched_equals_single(desc, lens, [[32, 27, 1][e % 3] for e in range(len(lens))], 3)
+
+
+@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_non_finite_row_reaches_only_rows_that_see_it(desc, bad):
+    """One input row that is not finite: the rows before it in its prefix, and the other prefixes, come out
+    as without it, bit for bit; the rows from it on are NaN. Rows at both ends of a 128-row block and of a
+    64-slot tile."""
+    lens = [300, 130, 257, 200, 64, 129]
+    rows = [0, 127, 128, 63, 64, 130, 199, 256, 299]
+    gpu = G.make_gpu(desc, G.to_cuda(data.make_weights(desc, 31)), max_seq=320, max_episodes=len(lens), max_rows=sum(lens),
+                     action_only=True)
+    gen = torch.Generator().manual_seed(5)
+    embeds = torch.randn(sum(lens), desc.d_model, generator=gen).mul_(0.5).to(torch.bfloat16).cuda()
+    ids, eps = [-1] * sum(lens), list(range(len(lens)))
+
+    def run(x):
+        _, logits = gpu.prefill(eps, x, ids, lens, want_logits=True)
+        # what the second layer wrote to the cache: the first layer's attention is in it
+        return logits.cpu(), [[gpu.read_kv(e, 1, which, 0, lens[e]) for which in (0, 1)] for e in eps]
+
+    good, kv = run(embeds)
+    assert torch.isfinite(good).all()
+    for e, row in [(0, r) for r in rows] + [(2, 255), (3, 198)]:
+        if row >= lens[e]:
+            continue
+        x = embeds.clone()
+        x[sum(lens[:e]) + row, 3] = bad
+        logits, got = run(x)
+        for other in eps:
+            first_bad = row if other == e else lens[other]
+            for which in (0, 1):
+                assert torch.equal(got[other][which][:first_bad], kv[other][which][:first_bad]), (e, row, other)
+                assert torch.isnan(got[other][which][first_bad:]).all(), (e, row, other)
+            if other != e:
+                assert torch.equal(logits[other], good[other])
+        assert torch.isnan(logits[e]).all()
+    gpu.close()
