@@ -1,7 +1,9 @@
-"""Attention of launches with many row blocks (batched prefill, batched verification) against the same
-episodes taken one at a time, whose few-row kernel the oracle tests pin; one episode against the
-oracle itself. Row counts sit at the edges of the 32- and 64-row blocks and of the 32-key tiles;
-the episode counts give launches of 32-row and of 64-row blocks."""
+"""Attention of launches with many rows (batched prefill, batched verification: blocks of 128 rows of one
+episode, key tiles of 64 slots in two buffers) against the same episodes taken one at a time, and some
+of them against the oracle itself. Episodes taken alone have at most 96 (32-row block, head) pairs and so
+run the few-row kernel, which the oracle tests pin. Row counts sit at the edges of the 32- and 128-row blocks
+and of the key tiles, with up to six tiles, so that both buffers are reused twice; trees of 128 rows
+start before, on and after a tile edge, so that their masks lie across one to three tiles."""
 import random
 
 import pytest
@@ -63,6 +65,15 @@ def test_batched_rows_equal_single_episodes(desc, n_ep):
     edges = [65, 31, 97, 64, 33, 128, 96, 129, 63, 127]
     lens = [edges[i % len(edges)] if n_ep == 60 or i % 2 == 0 else 70 + i for i in range(n_ep)]
     _batched_equals_single(desc, lens, [[27, 40, 65][e % 3] for e in range(n_ep)], n_ep)
+
+
+# prefixes of two and three row blocks and four to six key tiles; trees as wide as they get: the masks' upper
+# half, first bits at every kind of offset within a tile
+@pytest.mark.parametrize("desc", DESCS, ids=["head_dim64", "head_dim128"])
+def test_long_prefixes_and_wide_trees(desc):
+    lens = [255, 256, 257, 320, 319, 321, 191, 192, 193, 383, 128, 64, 63, 200]
+    rows = [128, 128, 128, 128, 65, 127, 128, 33, 97, 64, 128, 128, 128, 1]
+    _batched_equals_single(desc, lens, rows, 17, max_seq=520, oracle_eps=(2, 5, 9))
 
 
 # 75 to 96 (row block, head) pairs: the few-row kernel with one slice; a block of one row, a full one and
