@@ -546,7 +546,8 @@ row_attention_kernel(const EpArgs ea, const Args a) {
   const float *kbase = a.cache + (size_t)ea.eps[ei] * a.ep_stride + (size_t)h * DH;
   const float *vbase = kbase + (size_t)a.max_seq * hd;
 
-  if (tid == TC_THREADS - 1) s_clean = a.err[SV_NON_FINITE_V];
+  int flag = 0;
+  if (tid == TC_THREADS - 1) flag = a.err[SV_NON_FINITE_V];     // (in flight with the row tables)
   // last slot that any row sees: every warp finds it for itself
   int kmax = 0;
   {
@@ -570,6 +571,7 @@ row_attention_kernel(const EpArgs ea, const Args a) {
   for (int o = 16; o > 0; o >>= 1) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
   kmax = min(kmax, a.max_seq);
   const int tiles = (kmax + TC_KEYS - 1) / TC_KEYS;
+  if (tid == TC_THREADS - 1) s_clean = flag;
 
   // the loaders' first tile is on its way while the others prepare the queries
   const int lt = tid - 128;
