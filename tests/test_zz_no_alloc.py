@@ -60,3 +60,35 @@ def test_static_scratch_gemm_asynchronous_then_status():
     assert B.lib.specvla_gemm_static_status(B._stream()) == 0
     want = B.gemm(x, w).cpu().double()
     assert (y.cpu().double() - want).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
+
+
+def test_static_scratch_gemm_in_a_captured_graph():
+    """Two products in one captured graph (the second reads the first's result; both use the one
+    array), replayed with new operands: as the same two calls outside."""
+    import ctypes as C
+    from paper_2507_22424_b200 import binding as B
+    T, N, K = 27, 1024, 520
+    x, w = _case(51, T, N, K)
+    _, w2 = _case(52, 8, 512, N)
+    y, z = torch.empty(T, N, device="cuda"), torch.empty(T, 512, device="cuda")
+
+    def both():
+        for a, b, c in ((x, w, y), (y, w2, z)):
+            rc = B.lib.specvla_gemm_static(C.c_void_p(a.data_ptr()), C.c_void_p(b.data_ptr()), C.c_void_p(c.data_ptr()),
+                                           a.shape[0], b.shape[0], a.shape[1], 0, B._stream())
+            assert rc == 0
+
+    both()                                                  # the device's first call is outside the capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        both()
+    for seed in (53, 54, 55):
+        x.copy_(_case(seed, T, N, K)[0])
+        y.fill_(float("nan"))
+        z.fill_(float("nan"))
+        for _ in range(3):                                  # replays back to back share the array
+            graph.replay()
+        assert B.lib.specvla_gemm_static_status(B._stream()) == 0
+        want = B.gemm(B.gemm(x, w), w2)
+        assert torch.equal(z, want)
