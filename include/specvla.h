@@ -71,7 +71,7 @@ typedef struct {
                          * the LM head are quantised to int8, per output row, symmetric: scale =
                          * max|w| / 127 (1 for a zero row), code = round-half-even(w / scale) in
                          * [-127, 127], both in float32; the kernels stream the codes (half the bytes),
-                         * expand them to bf16 in shared memory and apply the scale to the accumulator.
+                         * expand them to bf16 in tensor memory and apply the scale to the accumulator.
                          * Embedding, norms and the draft model (with the original LM-head rows it
                          * scores with) are not quantised. The paper does not specify its scheme. */
 } specvla_model_desc;
@@ -244,8 +244,8 @@ int specvla_score_tree(specvla_ctx *ctx, int n_ep, const int *episodes, const sp
                        int *greedy_out, void *stream);
 
 /* Whole chunk (Algorithm 1): prefill, then draft -> verify -> accept until every episode has
- * n_tokens tokens; the result is clipped to n_tokens. One stream synchronisation per
- * iteration (the accepted length decides termination).
+ * n_tokens tokens; the result is clipped to n_tokens. One stream synchronisation per chunk where
+ * the loop runs on the device (SPECVLA_OPT_DEVICE_LOOP), else one per iteration.
  *   tokens_out   host [n_ep][n_tokens]
  *   actions_out  host [n_ep][n_tokens] bin centres in [-1, 1] (256 uniform bins), may be NULL
  *   stats        may be NULL */

@@ -32,8 +32,9 @@ constexpr int KT = 32;            // key slots per tile
 constexpr int THREADS = 256;      // 8 warps x 4 rows
 constexpr int MAX_SPLITS = 8;         // key slices per row block = cluster size (8: the portable limit)
 // (32-row block, head) pairs up to which a launch takes the few-row kernel: up to 64 rows of 32 heads
-// its slices are what fills the SMs; at 96 rows it measured 21.7 us against 24 for 128-row blocks,
-// which one episode has 32 of, at 128 rows 23.3 against 22.5.
+// its slices are what fills the SMs. Above, 128-row blocks, which one episode has 32 of, catch up: a
+// verification of 96 rows here and of 97 rows there takes 4.30 / 4.33 ms against 64 slots, 4.60 / 4.62
+// against 290 and 4.97 / 4.93 against 600; a layer's attention at 128 rows 23.3 us here, 22.5 there.
 constexpr int FEW_CTAS = 96;
 constexpr int MAX_SPLIT_CTAS = 148;   // CTAs of a launch that uses more than one key slice
 

@@ -3,7 +3,8 @@
 // A B200 SM can pull well over 100 GB/s through TMA, so ~64 streaming CTAs already saturate
 // HBM: there is no need to spread a matrix over all 148 SMs. Every GEMM of the decoder is
 // therefore cut into whole tiles first (LM head: 126 tiles = 126 CTAs, gate/up: 86, each
-// finishing its tile straight from TMEM with the fused epilogue), and only matrices with few
+// finishing its own tile: gate/up from TMEM, the others through a partial tile in shared
+// memory), and only matrices with few
 // tiles are split along K as well: the S (<= 8) CTAs that share a tile form one thread-block
 // cluster, CTA r streams K blocks [r KB / S, (r + 1) KB / S) through the TMA ring / tcgen05
 // pipeline, drops its fp32 partial tile into its own shared memory, and after one cluster
@@ -55,10 +56,10 @@ __device__ __forceinline__ void cluster_sync_all() {
 // tensor memory, where the MMAs read them as their A operand: a thread owns a weight row (64 codes
 // in from shared memory, 32 columns of bf16 pairs out). Shared memory then carries per unit only
 // the codes (written once, read once) and X: 56 KB at 32 rows, against 152 KB for an image expanded
-// in shared memory, whose three 32 KB buffers, block barriers and proxy fences bounded the kernel: a verification step
-// of 27 rows takes 3.23 ms instead of 4.26, of 8 rows 3.03 instead of 4.03, of 100 rows 5.71 instead
-// of 6.07. What is left over the bf16 weights' 3.00 ms is the chain of a unit: codes landed, 0.4 us
-// of expansion, MMAs, commit.
+// in shared memory, whose three 32 KB buffers, block barriers and proxy fences bounded the kernel: a
+// verification call of 27 rows takes 3.19 ms instead of 4.45, of 8 rows 3.04 instead of 4.23, of 97 rows
+// 5.63 instead of 6.16. What is left over the bf16 weights' 2.98 ms is the chain of a unit: codes landed,
+// 0.4 us of expansion, MMAs, commit.
 // TMEM: two accumulators of 2 TN columns, then q8_expanded(TN) buffers of 64 columns (two halves of
 // 128 rows x 64 K); 128 rows would leave no room for any, so Q8 chunks are at most 96 rows.
 // The codes have a ring of their own, free as soon as they are in registers; the X slot of a unit
@@ -790,7 +791,7 @@ inline cudaError_t launch_tq(const CUtensorMap &tmW, const CUtensorMap &tmX, con
   cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, gemm_ck_kernel<TN, MODE, Q8>, tmW, tmX, tmXtail, ea, KB, err);
 }
-// int8 weights (ea.wq8) take the instantiation that expands the codes in shared memory; the draft
+// int8 weights (ea.wq8) take the instantiation that expands the codes in tensor memory; the draft
 // scoring mode never runs on quantised weights.
 template <int TN, int MODE>
 inline cudaError_t launch_tm(const CUtensorMap &tmW, const CUtensorMap &tmX, const CUtensorMap &tmXtail,
@@ -874,7 +875,9 @@ inline int slices_for(int units, int KB, const ClusterFit &fit) {
 // instantiation, and chunk count and K slices are chosen together by a cost estimate in SM
 // clocks: waves x (fixed part of a CTA + its K blocks x clocks per K block), where a K block of tn
 // rows costs 512 + 6 tn clocks (what its 64 KB + 768 tn bytes of shared-memory traffic take at
-// 128 bytes per clock; the MMAs themselves need 8 tn).
+// 128 bytes per clock; the MMAs themselves need 8 tn). Fitted on a kernel that issued its MMAs under a
+// one-lane branch; the current one takes about 800 clocks at 80 rows, where this counts 992. int8
+// launches, whose shared-memory traffic is another, use the same estimate.
 struct RowPlan {
   int chunks, chunk_rows, tn_chunk, tn_tail, S;
 };

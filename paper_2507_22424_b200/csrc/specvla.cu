@@ -377,7 +377,7 @@ cudaLaunchConfig_t launch_cfg(dim3 grid, dim3 block, cudaStream_t st, cudaLaunch
   } while (0)
 
 // One GEMM over R rows of A against W with the fused epilogue described by `ea` (mode and
-// outputs; the row range is filled in here): one launch, 128 rows per CTA.
+// outputs; the row range is filled in here): one launch, up to 128 rows per CTA (int8 weights: 96).
 // next: the matrix of the GEMM that will follow (its head is prefetched into L2), or NULL.
 int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs ea, cudaStream_t st, int cls,
          const WMat *next = nullptr, bool next_swiglu = false) {
@@ -395,7 +395,7 @@ int gemm(specvla_ctx *ctx, const XBuf &A, const WMat &W, int R, gemm_tc::EpiArgs
   const bool prof = (ctx->prof_mask & ctx->phase) && 2 * (ctx->prof_used + 1) <= (int)ctx->prof_ev.size();
   if (prof) CU(cudaEventRecord(ctx->prof_ev[2 * ctx->prof_used], st));
   const gemm_ck::RowPlan plan = gemm_ck::plan_rows(R, tiles, KB, ctx->fit, W.q8 != nullptr);
-  const int chunks = plan.chunks, S = plan.S;
+  const int S = plan.S;
   ea.row0 = 0;
   ea.T = R;
   ea.chunk_rows = plan.chunk_rows;
