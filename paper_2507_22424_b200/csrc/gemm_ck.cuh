@@ -57,9 +57,13 @@ __device__ __forceinline__ void cluster_sync_all() {
 // in from shared memory, 32 columns of bf16 pairs out). Shared memory then carries per unit only
 // the codes (written once, read once) and X: 56 KB at 32 rows, against 152 KB for an image expanded
 // in shared memory, whose three 32 KB buffers, block barriers and proxy fences bounded the kernel: a
-// verification call of 27 rows takes 3.19 ms instead of 4.45, of 8 rows 3.04 instead of 4.23, of 97 rows
-// 5.63 instead of 6.16. What is left over the bf16 weights' 2.98 ms is the chain of a unit: codes landed,
-// 0.4 us of expansion, MMAs, commit.
+// verification call of 27 rows took 3.19 ms instead of 4.45, of 8 rows 3.04 instead of 4.23, of 97 rows
+// 5.63 instead of 6.16. A unit then took a CTA 0.45 us at every width up to 32 rows, the two sets of warps
+// of the epilogue taking turns; a third set (below) makes that 0.43 (27 rows 3.22 -> 3.11 ms, one row
+// 3.01 -> 2.89, 60 rows 3.75 -> 3.68). A fourth set, six expanded buffers instead of four, and copies of
+// a sixteenth of the codes change nothing more; with the conversion left out a unit takes 0.35 us, without the
+// stores to TMEM 0.30: what bounds it is instructions, two logical operations and a subtraction per two
+// codes, before the MMAs (0.14 us) and their hand-over.
 // TMEM: two accumulators of 2 TN columns, then q8_expanded(TN) buffers of 64 columns (two halves of
 // 128 rows x 64 K); 128 rows would leave no room for any, so Q8 chunks are at most 96 rows.
 // The codes have a ring of their own, free as soon as they are in registers; the X slot of a unit
@@ -73,7 +77,11 @@ __host__ __device__ constexpr int q8_x_bytes(int TN) { return 2 * q8_rows(TN) * 
 __host__ __device__ constexpr int q8_smem_bytes(int TN) {
   return Q8_STAGES * Q8_CODE_BYTES + q8_expanded(TN) * q8_x_bytes(TN) + 1024 + 256;
 }
-__host__ __device__ constexpr int ck_threads(bool Q8) { return Q8 ? THREADS + 32 : THREADS; }
+// Sets of four warps that expand, in turn: the two of the epilogue and up to 64 rows a third that does
+// nothing else. (Its threads leave 128 registers for each; long tiles need 148 to 163, and have two expanded
+// buffers only.)
+__host__ __device__ constexpr int q8_sets(int TN) { return TN > 64 ? 2 : 3; }
+__host__ __device__ constexpr int ck_threads(int TN, bool Q8) { return Q8 ? THREADS + 32 + 128 * (q8_sets(TN) - 2) : THREADS; }
 __host__ __device__ constexpr int ck_acc_width(int TN, bool Q8) { return Q8 ? 2 * q8_rows(TN) : acc_width(TN); }
 __host__ __device__ constexpr int ck_tmem_cols(int TN, bool Q8) {
   return Q8 ? 512 : (2 * acc_width(TN) < 32 ? 32 : 2 * acc_width(TN));
@@ -88,7 +96,7 @@ __device__ __forceinline__ uint32_t codes_to_bf16x2(uint32_t w) {
 
 // EpiArgs as in gemm_tc: the mode is a template parameter. KB = K blocks per tile.
 template <int TN, int MODE, bool Q8>
-__global__ void __launch_bounds__(ck_threads(Q8), 1)
+__global__ void __launch_bounds__(ck_threads(TN, Q8), 1)
 gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                const __grid_constant__ CUtensorMap tmXtail, const EpiArgs ea, const int KB,
                int *__restrict__ err) {
@@ -322,9 +330,11 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // ------------------------------------------------------------------ epilogue, part 1:
     // accumulator -> this CTA's partial tile P[t][256] in shared memory (the ring is idle by then)
     grid_dep_wait();
-    const int q = warp & 3, wp = (warp - 2) >> 2;
+    constexpr int SETS = q8_sets(TN);
+    const bool extra = Q8 && warp > 10;                  // a warp of the third set (Q8)
+    const int q = warp & 3, wp = extra ? 2 : (warp - 2) >> 2;
     const int et = threadIdx.x - 64;
-    if (et < T) {
+    if (et < T && !extra) {
       float sc = 1.f;
       if (ea.ssq_in) {
         float ss = 0.f;
@@ -344,7 +354,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const int p2_rg = p2_swiglu ? et >> 5 : et >> 6, p2_RG = p2_swiglu ? 8 : 4;
     const int p2_n = p2_swiglu ? tile * 128 + (et & 31) * 4 : tile * BM + (et & 63) * 4;
     const int p2_t0 = rank + p2_rg * S, p2_t1 = p2_t0 + p2_RG * S;
-    if (MODE == EPI_RESID && ea.accumulate && p2_n < ea.N) {
+    if (MODE == EPI_RESID && ea.accumulate && p2_n < ea.N && !extra) {
       if (p2_t0 < T) xpre0 = *reinterpret_cast<const float4 *>(ea.x + (size_t)(row0 + p2_t0) * ea.N + p2_n);
       if (p2_t1 < T) xpre1 = *reinterpret_cast<const float4 *>(ea.x + (size_t)(row0 + p2_t1) * ea.N + p2_n);
     }
@@ -357,8 +367,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     }
     if (Q8) {
-      // int8 -> bf16 expansion of every unit as it lands. The four warps of a set (wp) take every second
-      // unit, a warp the lanes of quarter q of both halves: two units are in expansion at once. The
+      // int8 -> bf16 expansion of every unit as it lands. The sets of four warps (wp) take the units in
+      // turn, a warp the lanes of quarter q of both halves: SETS units are in expansion at once. The
       // codes of the set's next unit are read while the stores of this one drain.
       const uint32_t trow = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(2 * AW);
       const uint32_t crow = base + (uint32_t)((q * 32 + lane) * 16);
@@ -375,7 +385,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       };
       bool ok = wp >= n_units || fetch_codes(wp);
       ok = __all_sync(0xffffffffu, ok);
-      for (int it = wp; ok && it < n_units; it += 2) {
+      for (int it = wp; ok && it < n_units; it += SETS) {
         __syncwarp();                                            // (a vote alone orders no memory)
         if (lane == 0) mbar_arrive(empty_bar(it % STAGES));      // every lane has read its codes
         const int e = it % NE, use = it / NE;
@@ -393,7 +403,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           }
           tc_st32(trow + (uint32_t)(e * 64 + h * 32), o);
         }
-        const bool got = it + 2 < n_units ? fetch_codes(it + 2) : true;
+        const bool got = it + SETS < n_units ? fetch_codes(it + SETS) : true;
         tc_wait_st();
         tc_fence_before();
         __syncwarp();
@@ -402,9 +412,9 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
       if (!ok && lane == 0) fail(SV_ERR_WAIT_FULL);
       __syncwarp();
-      epi_barrier();
     }
-    bool have = n_units > 0;
+    // (Q8: the accumulator is complete when every set has read its codes, so the partial tile may take their place)
+    bool have = n_units > 0 && !extra;
     if (have) {
       // one thread polls and the others sleep at the barrier (256 polling threads cost power and
       // shared-memory cycles for the whole stream)
@@ -428,7 +438,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
     const uint32_t tadr = tmem_base + ((uint32_t)(q * 32) << 16);
     const int col = q * 32 + lane;                       // column within a 128-column half
-    if (direct && have) {
+    if (extra) {
+    } else if (direct && have) {
       // A thread has gate and up of its column in the same TMEM lane, so an unsplit tile is finished
       // from registers. Two neighbouring lanes exchange a value each per pair of rows, so that both
       // store two columns of one row. (Prefill of 16 x 296 rows 112.6 -> 111.7 ms, of 290 rows 8.46 ->
@@ -540,13 +551,17 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       if (TN == MAX_T && S == 1) return *reinterpret_cast<const float4 *>(P_own + off);
       float4 p[MAX_S];
 #pragma unroll
-      for (int sl = 0; sl < MAX_S; sl++)
+      for (int sl = 0; sl < MAX_S; sl++) {
+        // (Or what p held before would be kept in registers: 134 instead of 96 for the QKV mode of the wide
+        // Q8 block, which has 128. Where registers are not short it costs time: 128 bf16 rows +1.6 %.)
+        if (Q8) p[sl] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (sl < S) {
           // rank sl's copy of the same shared-memory address (mapped on the spot: an array of
           // eight mapped pointers would cost sixteen registers)
           const float *P = S == 1 ? P_own : cluster.map_shared_rank(const_cast<float *>(P_own), (unsigned)sl);
           p[sl] = *reinterpret_cast<const float4 *>(P + off);
         }
+      }
       float4 acc = p[0];
 #pragma unroll
       for (int sl = 1; sl < MAX_S; sl++)
@@ -777,7 +792,7 @@ inline cudaError_t launch_tq(const CUtensorMap &tmW, const CUtensorMap &tmX, con
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles * S, (ea.T + ea.chunk_rows - 1) / ea.chunk_rows);
-  cfg.blockDim = dim3(ck_threads(Q8));
+  cfg.blockDim = dim3(ck_threads(TN, Q8));
   cfg.dynamicSmemBytes = SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];

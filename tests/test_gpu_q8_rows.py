@@ -45,3 +45,22 @@ def test_code_ring_is_refilled(n_rows):
     # a unit whose codes were overwritten moves every logit by far more than rounding does
     assert tally.accepts == 1 and tally.caches == 1 and tally.max_logit_err < 2e-4, tally.max_logit_err
     gpu.close()
+
+
+@pytest.mark.parametrize("k_blocks", [1, 2, 3])
+def test_fewer_units_than_expanding_sets(k_blocks):
+    """One to three K blocks per tile: some sets of expanding warps have no unit, or exactly one."""
+    desc = C.ModelDesc(n_layers=2, d_model=64 * k_blocks, n_heads=2, head_dim=64, d_ffn=64 * k_blocks, vocab=1024,
+                       action_base=768)
+    w = data.make_weights(desc, 6)
+    orc = SpecVLAOracle(desc, Q.quantize_target(w))
+    gpu = G.make_gpu(desc, G.to_cuda(w), max_seq=256, max_episodes=1, max_rows=256, action_only=True, weight_bits=8)
+    tally = G.Tally()
+    ids = torch.arange(40) * 7 % desc.action_base
+    embeds = torch.zeros(40, desc.d_model, dtype=torch.bfloat16)
+    ep, _, _ = G.prefill_both(orc, gpu, embeds.cuda(), ids, 0, tally, desc)
+    tok, par, dep = data.random_tree(27, desc, seed=k_blocks, max_depth=8, root_token=ep.root)
+    G.verify_both(orc, gpu, ep, Tree(tok, par, dep, [0.0] * 27), 40, tally, desc, where=f"q8.units({k_blocks})")
+    # a unit that was left out moves every logit by far more than rounding does (2e-4, as above)
+    assert tally.accepts == 1 and tally.caches == 1 and tally.max_logit_err < 2e-4, tally.max_logit_err
+    gpu.close()
