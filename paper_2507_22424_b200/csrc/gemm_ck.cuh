@@ -94,29 +94,42 @@ __device__ __forceinline__ uint32_t codes_to_bf16x2(uint32_t w) {
   return *reinterpret_cast<const uint32_t *>(&r);
 }
 
+// The long bf16 instantiation sizes its stages by the rows of its chunks (a tail has no more), and has four
+// of them up to 88 rows, three above: the most that fit beside the kernel's static shared memory. Three
+// stages of 64 KB, whatever the rows, did not cover the latency of the weights at 65 to 88 rows, where the
+// MMAs take less than they do: a verification step of 70 rows 4.16 -> 4.01 ms. (Rings of their own for
+// weights and X, four to six slots of one and two to four of the other, cost a second commit and a second
+// wait per K block: 96 rows -1 %, a prefill of 290 rows +3.5 %.)
+constexpr int LONG_STAGES = 4, LONG_RING = 216 * 1024;
+__host__ __device__ constexpr int long_stages(int tn) { return LONG_STAGES * stage_bytes(tn) <= LONG_RING ? LONG_STAGES : 3; }
+__host__ __device__ constexpr int long_smem_bytes(int tn) { return long_stages(tn) * stage_bytes(tn) + 1024 + 256; }
+
 // EpiArgs as in gemm_tc: the mode is a template parameter. KB = K blocks per tile.
 template <int TN, int MODE, bool Q8>
 __global__ void __launch_bounds__(ck_threads(TN, Q8), 1)
 gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                const __grid_constant__ CUtensorMap tmXtail, const EpiArgs ea, const int KB,
                int *__restrict__ err) {
-  constexpr int STAGES = Q8 ? Q8_STAGES : stages_of(TN);
-  constexpr int STAGE = Q8 ? Q8_CODE_BYTES : stage_bytes(TN);
+  // stages and their size: the long bf16 instantiation's follow from its rows
+  constexpr bool LONG = TN == MAX_T && !Q8;
+  constexpr int MAX_STAGES = Q8 ? Q8_STAGES : LONG ? LONG_STAGES : stages_of(TN);
+  const int STAGES = LONG ? long_stages(ea.tn_chunk) : MAX_STAGES;
+  const int STAGE = Q8 ? Q8_CODE_BYTES : LONG ? stage_bytes(ea.tn_chunk) : stage_bytes(TN);
   constexpr int NE = Q8 ? q8_expanded(TN) : 1;                // expanded buffers in TMEM
-  constexpr int RING_BYTES = STAGES * STAGE + (Q8 ? NE * q8_x_bytes(TN) : 0);
+  const int RING_BYTES = STAGES * STAGE + (Q8 ? NE * q8_x_bytes(TN) : 0);
   constexpr int AW = ck_acc_width(TN, Q8);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t bars = base + RING_BYTES;
   auto full_bar = [&](int s) { return bars + 8u * s; };
-  auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
-  const uint32_t tfull_bar = bars + 8u * (2 * STAGES);
-  const uint32_t tmem_slot = bars + 8u * (2 * STAGES + 1);
+  auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
+  const uint32_t tfull_bar = bars + 8u * (2 * MAX_STAGES);
+  const uint32_t tmem_slot = bars + 8u * (2 * MAX_STAGES + 1);
   // Q8: expanded buffer e holds the bf16 image of a unit (conv) / has been read by its MMAs, like X slot e (efree);
   // X slot e, behind the codes, holds the unit's X (xfull)
-  auto conv_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + e); };
-  auto efree_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + NE + e); };
-  auto xfull_bar = [&](int e) { return bars + 8u * (2 * STAGES + 2 + 2 * NE + e); };
+  auto conv_bar = [&](int e) { return bars + 8u * (2 * MAX_STAGES + 2 + e); };
+  auto efree_bar = [&](int e) { return bars + 8u * (2 * MAX_STAGES + 2 + NE + e); };
+  auto xfull_bar = [&](int e) { return bars + 8u * (2 * MAX_STAGES + 2 + 2 * NE + e); };
   auto x_slot = [&](int e) { return base + (uint32_t)(STAGES * STAGE + e * q8_x_bytes(TN)); };
   __shared__ float s_scale[MAX_T];
   __shared__ int s_pos[MAX_T], s_slot[MAX_T], s_ep[MAX_T];
@@ -172,9 +185,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint64_t pol_w = policy_evict_first();
   // test hook: the K block that is never loaded (-1: none)
   const int withheld = ea.withhold_unit - 1;
-  auto load_w = [&](int it) {
+  auto load_w = [&](int it, int st) {
     if (it == withheld) return;
-    const int st = it % STAGES;
     const uint32_t sW = base + st * STAGE;
     mbar_expect_tx(full_bar(st), stage_tx);
     if (Q8) {
@@ -209,7 +221,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     grid_dep_launch();
-    for (int it = 0; it < npre; it++) load_w(it);
+    for (int it = 0; it < npre; it++) load_w(it, it);
   }
   if (warp == 1) {
     tc_alloc(tmem_slot, ck_tmem_cols(TN, Q8));
@@ -253,7 +265,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         break;
       }
       if (lead) {
-        load_w(it);
+        load_w(it, st);
         if (!Q8) load_x(it, st);
       }
       __syncwarp();
@@ -374,7 +386,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const uint32_t crow = base + (uint32_t)((q * 32 + lane) * 16);
       uint32_t c[32];
       auto fetch_codes = [&](int it) {
-        const int st = it % STAGES, rnd = it / STAGES;
+        const int st = it % MAX_STAGES, rnd = it / MAX_STAGES;
         if (!mbar_wait(full_bar(st), rnd & 1, ea.wait_ns)) return false;
 #pragma unroll
         for (int k = 0; k < 8; k++)
@@ -387,7 +399,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       ok = __all_sync(0xffffffffu, ok);
       for (int it = wp; ok && it < n_units; it += SETS) {
         __syncwarp();                                            // (a vote alone orders no memory)
-        if (lane == 0) mbar_arrive(empty_bar(it % STAGES));      // every lane has read its codes
+        if (lane == 0) mbar_arrive(empty_bar(it % MAX_STAGES));      // every lane has read its codes
         const int e = it % NE, use = it / NE;
         if (use > 0) ok = mbar_wait(efree_bar(e), (use - 1) & 1, ea.wait_ns);
         ok = __all_sync(0xffffffffu, ok);
@@ -787,13 +799,14 @@ template <int TN, int MODE, bool Q8>
 inline cudaError_t launch_tq(const CUtensorMap &tmW, const CUtensorMap &tmX, const CUtensorMap &tmXtail,
                              const EpiArgs &ea, int tiles, int KB, int S, int *err, cudaStream_t st, bool pdl) {
   // per device and cheap: set on every launch, so that every device of the process has it
-  constexpr int SMEM = Q8 ? q8_smem_bytes(TN) : smem_bytes(TN);
+  // (the attribute is the most that any launch asks for: launches of other sizes may be made at the same time)
+  constexpr int SMEM = Q8 ? q8_smem_bytes(TN) : TN == MAX_T ? LONG_RING + 1024 + 256 : smem_bytes(TN);
   cudaError_t e = cudaFuncSetAttribute(gemm_ck_kernel<TN, MODE, Q8>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles * S, (ea.T + ea.chunk_rows - 1) / ea.chunk_rows);
   cfg.blockDim = dim3(ck_threads(TN, Q8));
-  cfg.dynamicSmemBytes = SMEM;
+  cfg.dynamicSmemBytes = !Q8 && TN == MAX_T ? long_smem_bytes(ea.tn_chunk) : SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;

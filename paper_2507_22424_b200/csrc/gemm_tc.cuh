@@ -41,8 +41,8 @@ __host__ __device__ constexpr int stage_bytes(int TN) { return W_STAGE_BYTES + 2
 // between two GEMMs can be resident next to a GEMM CTA while it prefetches weights (a fifth stage
 // measured the same). At 64 rows a stage is 48 KB and three of them do not cover the load latency:
 // four take a verification step of 64 rows from 3.77 to 3.59 ms, a prefill of 34 rows from 3.53 to
-// 3.35 ms. At 128 rows (prefill) a stage is 64 KB and three are what there is room for.
-__host__ __device__ constexpr int stages_of(int TN) { return TN > 64 ? 3 : TN > 32 ? 4 : RING_BUDGET / stage_bytes(TN); }
+// 3.35 ms. (The 128-row instantiation: gemm_ck::long_stages.)
+__host__ __device__ constexpr int stages_of(int TN) { return TN > 32 ? 4 : RING_BUDGET / stage_bytes(TN); }
 __host__ __device__ constexpr int smem_bytes(int TN) { return stages_of(TN) * stage_bytes(TN) + 1024 + 256; }
 // Both limbs of X form ONE MMA operand (N = 2 TN: hi rows, then lo rows; 256 at most, the
 // largest N of an M = 128 MMA), which reads the weight operand from shared memory once for

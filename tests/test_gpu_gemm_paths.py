@@ -32,6 +32,19 @@ def test_widths_between_33_and_64_rows(T):
     _check(T, 1000, 520, True)
 
 
+# the long instantiation sizes its ring by the rows: four stages up to 88, three above; 17 K blocks go
+# through it, unsplit, so that every stage is refilled
+@pytest.mark.parametrize("T", [65, 72, 80, 81, 88, 89, 96, 128])
+def test_ring_sizes_of_long_tiles(T):
+    _check(T, 20480, 1032, True)
+
+
+# several chunks: 88-row chunks of four stages with a shorter tail
+@pytest.mark.parametrize("T", [170, 176])
+def test_ring_sizes_of_several_chunks(T):
+    _check(T, 4096, 2056, True)
+
+
 def test_operand_off_a_16_byte_boundary():
     """The split takes X four values at a time only where it starts on 16 bytes."""
     from paper_2507_22424_b200.binding import gemm
