@@ -57,3 +57,29 @@ def test_a_wait_limit_covers_the_product_alone(T, N, K):
         assert B.lib.specvla_gemm_fault_test(200_000, -1) == 0          # no K block is withheld
         y = B.gemm(x, w)                                                # (raises on a timeout)
     assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
+
+
+def test_status_belongs_to_the_calling_thread():
+    """Products from several threads on streams of their own: each reads its own status and result."""
+    import threading
+    from paper_2507_22424_b200.binding import gemm_prepacked, pack_weights
+    g = torch.Generator().manual_seed(3)
+    w = torch.randn(256, 264, generator=g).to(torch.bfloat16).cuda()
+    packed = pack_weights(w)
+    xs = [torch.randn(n, 264, generator=g).cuda() for n in (1, 9, 33)]
+    want = [gemm_prepacked(x, packed, 256) for x in xs]
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(i):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(50):
+                if not torch.equal(gemm_prepacked(xs[i], packed, 256), want[i]):
+                    bad.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(xs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
