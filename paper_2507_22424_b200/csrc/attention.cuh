@@ -429,8 +429,9 @@ tree_attention_kernel(const EpArgs ea, const Args a) {
       a.out[a.out_plane + idx] = __float2bfloat16(v - __bfloat162float(hi));
     }
   }
-  // nobody leaves while a peer may still be reading its shared memory
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // nobody leaves while a peer may still be reading its shared memory (relaxed: nothing is handed over, and
+  // a releasing arrival would first wait for the output's stores)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
