@@ -35,7 +35,7 @@ WEIGHT_BYTES_PER_VERIFY = 32 * 404_750_336 + 256 * 4096 * 2
 
 # DRAM traffic of one gate/up launch at T = 27 from the ncu capture under profiles/ (bytes); to be
 # re-taken (or set to None) whenever gemm_ck.cuh changes.
-GATE_UP_DRAM_BYTES = 203_317_504 + 3_897_856
+GATE_UP_DRAM_BYTES = 203_070_976 + 3_492_096
 GATE_UP_DRAM_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of this launch at full size "
                        "(profiles/gemm_ck_verify_T27_ncu_full.md); the ~23 MB above the weights are the operand "
                        "and the L2 prefetch of the next GEMM's weights")
@@ -357,7 +357,7 @@ def int8_target(weights, desc, embeds, ids_host, P, shape, r, n_tok, steps=5):
     return dict(value=steps / (ms * 1e-3), unit=UNIT, verify_ms_per_step=ms_v / max(1, iters),
                 weight_bytes_per_step=WEIGHT_BYTES_FULL_HEAD // 2, lossless_vs_own_ar=bool(toks == ar), tokens=toks[0],
                 note="int8 codes are streamed at half the bytes and expanded to bf16 into tensor memory, where the "
-                     "tensor cores read them; the chain of a unit (expansion, hand-over, MMAs), not HBM, bounds this path")
+                     "tensor cores read them; the instructions of the expansion and its hand-overs, not HBM, bound this path")
 
 
 # --------------------------------------------------------------------------- CUDA arm
