@@ -1964,15 +1964,20 @@ int specvla_gemm_status(const void *scratch, void *stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int local = 0;
   volatile int *word = g_status_word.p ? g_status_word.p : &local;
-  if (g_status_word.p) {
+  // the kernel reads memory of the device that is current; scratch that lies elsewhere is copied
+  cudaPointerAttributes where = {};
+  int dev = -1;
+  bool sent = false;
+  if (g_status_word.p && cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&where, scratch) == cudaSuccess &&
+      where.type == cudaMemoryTypeDevice && where.device == dev) {
     cudaLaunchAttribute at;
     const cudaLaunchConfig_t cfg = launch_cfg(dim3(1), dim3(1), st, &at, true);
-    if (cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), g_status_word.p) != cudaSuccess) {
-      cudaGetLastError();
-      return SPECVLA_ERR_CUDA;
-    }
-  } else if (cudaMemcpyAsync(&local, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) {
-    return SPECVLA_ERR_CUDA;
+    sent = cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), g_status_word.p) == cudaSuccess;
+    if (!sent) cudaGetLastError();
+  }
+  if (!sent) {
+    word = &local;
+    if (cudaMemcpyAsync(&local, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return SPECVLA_ERR_CUDA;
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) return SPECVLA_ERR_CUDA;
   return *word == 0 ? SPECVLA_OK : SPECVLA_ERR_TIMEOUT;
