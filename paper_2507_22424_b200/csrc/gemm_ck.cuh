@@ -549,6 +549,11 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const int c4 = swiglu ? (et & 31) * 4 : (et & 63) * 4;    // first of the four columns within the tile
     const int n = swiglu ? tile * 128 + c4 : tile * BM + c4;
     const bool col_ok = n < ea.N;                             // N % 4 == 0: all four or none
+    // Peers' partial tiles are read only where something is stored that depends on them: the exit barrier
+    // below relies on it. (A scoring launch that returns no logits uses the columns of its id range alone.)
+    // The other threads read this CTA's own tile instead: a branch around the reads makes a verification
+    // call of 27 int8 rows 2 % slower (3.00 -> 3.06 ms), a prefill of 34 rows 0.5 %.
+    const bool used = col_ok && ((MODE != EPI_PLAIN && MODE != EPI_TOPK) || ea.out || (n + 3 >= ea.lo && n < ea.hi));
     const float *P_own = reinterpret_cast<const float *>(smem_raw + (base - smem_u32(smem_raw)));
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     float4 gain = make_float4(1.f, 1.f, 1.f, 1.f);
@@ -570,7 +575,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (sl < S) {
           // rank sl's copy of the same shared-memory address (mapped on the spot: an array of
           // eight mapped pointers would cost sixteen registers)
-          const float *P = S == 1 ? P_own : cluster.map_shared_rank(const_cast<float *>(P_own), (unsigned)sl);
+          const float *P = S == 1 ? P_own : cluster.map_shared_rank(const_cast<float *>(P_own), (unsigned)(used ? sl : rank));
           p[sl] = *reinterpret_cast<const float4 *>(P + off);
         }
       }
@@ -770,7 +775,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // This CTA has read all it needs from its peers: say so now, and wait for the peers' word only
   // before leaving (nobody leaves while a peer may still be reading its shared memory), so that
   // the barrier's latency passes behind the rest of the epilogue. Relaxed: the barrier hands nothing over,
-  // and what this CTA has read is in stores already issued. A releasing arrival makes every warp wait until
+  // and a value that was read from a peer has arrived, because a store that depends on it has been issued
+  // (`used` above: no such read is without one). A releasing arrival makes every warp wait until
   // the tile's stores to global memory are through, before a barrier that the peers wait for: verification of
   // 1 / 27 / 60 rows 2.73 / 2.99 / 3.54 ms with it here and in the few-row attention, 2.63 / 2.92 / 3.50 without.
   if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
