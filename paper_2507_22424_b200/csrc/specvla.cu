@@ -1843,6 +1843,15 @@ static __global__ void status_to_host_kernel(const int *status, int *host) {
   *host = *status;
 }
 
+// The same by a copy to the stack, which allocates nothing.
+static int status_by_copy(const void *scratch, cudaStream_t st) {
+  int word = 0;
+  if (cudaMemcpyAsync(&word, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return SPECVLA_ERR_CUDA;
+  return word == 0 ? SPECVLA_OK : SPECVLA_ERR_TIMEOUT;
+}
+
 // W (row-major) or Wp (repacked) is given, never both.
 static int gemm_entry(const float *X, const void *W, const void *Wp, float *Y, int T, int N, int K, void *scratch,
                       size_t scratch_bytes, void *stream) {
@@ -1942,7 +1951,7 @@ int specvla_gemm_static(const float *X, const void *W, float *Y, int T, int N, i
   void *scratch = reinterpret_cast<void *>(base);
   const int rc = specvla_gemm(X, W, Y, T, N, K, scratch, SPECVLA_STATIC_SCRATCH_BYTES, stream);
   if (rc != SPECVLA_OK || !wait) return rc;
-  return specvla_gemm_status(scratch, stream);
+  return status_by_copy(scratch, static_cast<cudaStream_t>(stream));
 }
 
 int specvla_gemm_static_status(void *stream) {
@@ -1955,29 +1964,25 @@ int specvla_gemm_static_status(void *stream) {
   }
   if (!addr) return SPECVLA_ERR_BAD_STATE;            // specvla_gemm_static has not run on this device
   const uintptr_t base = (reinterpret_cast<uintptr_t>(addr) + 1023) & ~(uintptr_t)1023;
-  return specvla_gemm_status(reinterpret_cast<const void *>(base), stream);
+  return status_by_copy(reinterpret_cast<const void *>(base), static_cast<cudaStream_t>(stream));
 }
 
 int specvla_gemm_status(const void *scratch, void *stream) {
   if (!scratch) return SPECVLA_ERR_INVALID_ARG;
   g_status_word.get();
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int local = 0;
-  volatile int *word = g_status_word.p ? g_status_word.p : &local;
   // the kernel reads memory of the device that is current; scratch that lies elsewhere is copied
   cudaPointerAttributes where = {};
   int dev = -1;
-  bool sent = false;
-  if (g_status_word.p && cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&where, scratch) == cudaSuccess &&
-      where.type == cudaMemoryTypeDevice && where.device == dev) {
-    cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = launch_cfg(dim3(1), dim3(1), st, &at, true);
-    sent = cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), g_status_word.p) == cudaSuccess;
-    if (!sent) cudaGetLastError();
-  }
-  if (!sent) {
-    word = &local;
-    if (cudaMemcpyAsync(&local, scratch, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return SPECVLA_ERR_CUDA;
+  if (!g_status_word.p || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&where, scratch) != cudaSuccess ||
+      where.type != cudaMemoryTypeDevice || where.device != dev)
+    return status_by_copy(scratch, st);
+  volatile int *word = g_status_word.p;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = launch_cfg(dim3(1), dim3(1), st, &at, true);
+  if (cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), g_status_word.p) != cudaSuccess) {
+    cudaGetLastError();
+    return status_by_copy(scratch, st);
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) return SPECVLA_ERR_CUDA;
   return *word == 0 ? SPECVLA_OK : SPECVLA_ERR_TIMEOUT;

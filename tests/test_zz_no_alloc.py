@@ -3,6 +3,10 @@
 a fixed array inside the library, so this checks that it gives what specvla_gemm gives with
 caller-allocated scratch, twice in a row on the shared array, and that it refuses shapes the
 array cannot hold. Collected last on purpose: a failure here cannot hide another test."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -92,3 +96,44 @@ def test_static_scratch_gemm_in_a_captured_graph():
         assert B.lib.specvla_gemm_static_status(B._stream()) == 0
         want = B.gemm(B.gemm(x, w), w2)
         assert torch.equal(z, want)
+
+
+# In a process of its own, where nothing else has mapped page-locked memory yet: the driver maps it from
+# /dev/zero, two megabytes at least for the first four bytes.
+ALLOCATES = """
+import threading
+import torch
+from paper_2507_22424_b200 import binding as B
+
+x = torch.randn(9, 264, device="cuda")
+w = torch.randn(256, 264, device="cuda").to(torch.bfloat16)
+y = torch.empty(9, 256, device="cuda")
+
+
+def page_locked():
+    return sorted(line.split()[0] for line in open("/proc/self/maps") if "/dev/zero" in line)
+
+
+def calls():
+    B.gemm_static(x, w, y)                                  # waits
+    assert B.lib.specvla_gemm_static_status(B._stream()) == 0
+
+
+rc = B.lib.specvla_gemm_static(x.data_ptr(), w.data_ptr(), y.data_ptr(), 9, 256, 264, 0, B._stream())
+assert rc == 0
+torch.cuda.synchronize()
+y.cpu()                                                     # the device and the copy path are set up
+before = page_locked()
+calls()
+thread = threading.Thread(target=calls)
+thread.start()
+thread.join()
+assert page_locked() == before, (before, page_locked())
+"""
+
+
+def test_static_gemm_allocates_no_page_locked_memory():
+    """A call that waits and the status call, on a thread's first use."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    done = subprocess.run([sys.executable, "-c", ALLOCATES], cwd=root, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr[-2000:]
