@@ -302,7 +302,9 @@ int specvla_gemm_fault_test(long long wait_limit_ns, int withhold_k_block);
 
 /* Synchronises `stream` and reports whether the specvla_gemm calls that used `scratch` ran
  * to completion: SPECVLA_ERR_TIMEOUT if a bounded device-side wait gave up (Y is then
- * undefined), SPECVLA_ERR_CUDA if the stream is in error, else SPECVLA_OK. */
+ * undefined), SPECVLA_ERR_CUDA if the stream is in error, else SPECVLA_OK. The first call in a CUDA
+ * context allocates 256 bytes of page-locked memory, which all threads share and which stay with
+ * the context; no later call allocates. */
 int specvla_gemm_status(const void *scratch, void *stream);
 
 /* specvla_gemm for callers that cannot allocate device memory: code running inside a CUDA

@@ -1815,29 +1815,79 @@ int specvla_pack_weights(const void *W, int N, int K, void *packed, size_t packe
   return cudaGetLastError() == cudaSuccess ? SPECVLA_OK : SPECVLA_ERR_CUDA;
 }
 
-// Where a thread's status read-backs land: four bytes of page-locked memory per thread, given back when it
-// ends. A kernel that is launched beside the GEMM and waits for it writes the word there: a call with 27 / 1 / 200
-// rows of 11008 / 4096 / 4096 takes 41.8 / 32.8 / 43.7 us, with an ordinary launch 44.5 / 34.8 / 46.1, with a
-// copy to page-locked memory 45.5 / 36.2 / 47.8, with a copy to the stack (staged by the driver) 47.3 / 38.0 /
-// 49.5. Without page-locked memory that last way serves.
-struct StatusWord {
-  int *p = nullptr;
-  bool tried = false;
-  void get() {
-    if (tried) return;
-    tried = true;
+// Driver calls of the status read-back, looked up once.
+struct DriverCalls {
+  decltype(&cuCtxGetCurrent) current = nullptr;
+  decltype(&cuCtxGetId) id = nullptr;
+  DriverCalls() {
+    current = reinterpret_cast<decltype(current)>(find("cuCtxGetCurrent"));
+    id = reinterpret_cast<decltype(id)>(find("cuCtxGetId"));
+  }
+  static void *find(const char *name) {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+};
+static const DriverCalls &driver_calls() {
+  static const DriverCalls calls;
+  return calls;
+}
+
+// Where status read-backs land: 64 page-locked words per CUDA context, allocated by its first read-back; a
+// call holds one while it waits. They are found by the context's id, which no later context gets, so words
+// that went with their context (cudaDeviceReset, cuCtxDestroy) are not touched again, and no thread owns or
+// frees any. Beyond 64 calls at a time or 16 contexts, or without page-locked memory, a call takes a copy.
+struct StatusWords {
+  unsigned long long ctx, taken;                     // owner's id; one bit per word
+  int *words;                                        // NULL: the allocation was refused
+};
+constexpr int STATUS_CONTEXTS = 16, STATUS_WORDS = 64;
+static std::mutex g_status_mutex;
+static StatusWords g_status_words[STATUS_CONTEXTS];
+static int g_status_contexts;
+
+// A free word of the current context, or NULL.
+static int *take_status_word() {
+  const DriverCalls &cu = driver_calls();
+  CUcontext ctx = nullptr;
+  unsigned long long id = 0;
+  if (!cu.current || !cu.id || cu.current(&ctx) != CUDA_SUCCESS || !ctx || cu.id(ctx, &id) != CUDA_SUCCESS) return nullptr;
+  std::lock_guard<std::mutex> lock(g_status_mutex);
+  int i = 0;
+  while (i < g_status_contexts && g_status_words[i].ctx != id) i++;
+  if (i == STATUS_CONTEXTS) return nullptr;
+  StatusWords &b = g_status_words[i];
+  if (i == g_status_contexts) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // (another thread may be capturing)
     cudaThreadExchangeStreamCaptureMode(&mode);
     void *m = nullptr;
-    if (cudaHostAlloc(&m, sizeof(int), cudaHostAllocPortable) == cudaSuccess) p = static_cast<int *>(m);
-    else cudaGetLastError();
+    if (cudaHostAlloc(&m, STATUS_WORDS * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+      m = nullptr;
+      cudaGetLastError();
+    }
     cudaThreadExchangeStreamCaptureMode(&mode);
+    b = {id, 0, static_cast<int *>(m)};
+    g_status_contexts++;
   }
-  ~StatusWord() {
-    if (p) cudaFreeHost(p);
-  }
-};
-static thread_local StatusWord g_status_word;
+  if (!b.words || b.taken == ~0ull) return nullptr;
+  const int w = __builtin_ctzll(~b.taken);
+  b.taken |= 1ull << w;
+  return b.words + w;
+}
+static void give_status_word(const int *word) {
+  std::lock_guard<std::mutex> lock(g_status_mutex);
+  for (int i = 0; i < g_status_contexts; i++)
+    if (g_status_words[i].words && word >= g_status_words[i].words && word < g_status_words[i].words + STATUS_WORDS)
+      g_status_words[i].taken &= ~(1ull << (word - g_status_words[i].words));
+}
+
+// A kernel that is launched beside the GEMM and waits for it writes the word there: a call with 27 / 1 / 200
+// rows of 11008 / 4096 / 4096 takes 41.8 / 32.8 / 43.7 us, with an ordinary launch 44.5 / 34.8 / 46.1, with a
+// copy to page-locked memory 45.5 / 36.2 / 47.8, with a copy to the stack (staged by the driver) 47.3 / 38.0 /
+// 49.5.
 static __global__ void status_to_host_kernel(const int *status, int *host) {
   pdl_wait();
   *host = *status;
@@ -1969,23 +2019,26 @@ int specvla_gemm_static_status(void *stream) {
 
 int specvla_gemm_status(const void *scratch, void *stream) {
   if (!scratch) return SPECVLA_ERR_INVALID_ARG;
-  g_status_word.get();
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the kernel reads memory of the device that is current; scratch that lies elsewhere is copied
   cudaPointerAttributes where = {};
   int dev = -1;
-  if (!g_status_word.p || cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&where, scratch) != cudaSuccess ||
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&where, scratch) != cudaSuccess ||
       where.type != cudaMemoryTypeDevice || where.device != dev)
     return status_by_copy(scratch, st);
-  volatile int *word = g_status_word.p;
+  int *word = take_status_word();
+  if (!word) return status_by_copy(scratch, st);
   cudaLaunchAttribute at;
   const cudaLaunchConfig_t cfg = launch_cfg(dim3(1), dim3(1), st, &at, true);
-  if (cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), g_status_word.p) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, status_to_host_kernel, static_cast<const int *>(scratch), word) != cudaSuccess) {
     cudaGetLastError();
+    give_status_word(word);
     return status_by_copy(scratch, st);
   }
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SPECVLA_ERR_CUDA;
-  return *word == 0 ? SPECVLA_OK : SPECVLA_ERR_TIMEOUT;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return SPECVLA_ERR_CUDA;     // (the kernel may yet write: the word stays taken)
+  const int status = *static_cast<volatile int *>(word);
+  give_status_word(word);
+  return status == 0 ? SPECVLA_OK : SPECVLA_ERR_TIMEOUT;
 }
 
 int specvla_profile(specvla_ctx *ctx, int enable) {

@@ -1,5 +1,10 @@
 """A stand-alone product that is refused fails alone: its error and the one-call test hook end with it."""
 import ctypes as C
+import os
+import subprocess
+import sys
+import threading
+import time
 
 import pytest
 import torch
@@ -61,7 +66,6 @@ def test_a_wait_limit_covers_the_product_alone(T, N, K):
 
 def test_status_belongs_to_the_calling_thread():
     """Products from several threads on streams of their own: each reads its own status and result."""
-    import threading
     from paper_2507_22424_b200.binding import gemm_prepacked, pack_weights
     g = torch.Generator().manual_seed(3)
     w = torch.randn(256, 264, generator=g).to(torch.bfloat16).cuda()
@@ -83,3 +87,68 @@ def test_status_belongs_to_the_calling_thread():
     for t in threads:
         t.join()
     assert not bad, bad
+
+
+def test_a_thread_may_end_inside_another_threads_capture():
+    """The end of a thread that has read a status makes no call that a capture forbids."""
+    from paper_2507_22424_b200 import binding as B
+    x, w, ref = _operands(9, 256, 264)
+    asked, end = threading.Event(), threading.Event()
+
+    def work():
+        B.gemm(x, w)
+        asked.set()
+        end.wait()
+
+    thread = threading.Thread(target=work)
+    thread.start()
+    asked.wait()
+    torch.cuda.synchronize()
+    y = torch.ones(8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        y.mul_(2)
+        end.set()
+        thread.join()
+        time.sleep(0.3)                                                 # (its thread-local objects go after the join)
+        y.add_(1)
+    graph.replay()
+    assert y.tolist() == [3.0] * 8
+
+
+# Contexts that come and go under one thread: each reads its own status, before and after the others.
+CONTEXTS = """
+import ctypes as C
+import torch
+from paper_2507_22424_b200 import binding as B
+
+cu = C.CDLL("libcuda.so.1")
+
+
+def ok(rc):
+    assert rc == 0, rc
+
+
+x = torch.ones(9, 264, device="cuda")
+w = torch.ones(256, 264, device="cuda", dtype=torch.bfloat16)
+primary = C.c_void_p()
+for _ in range(20):                                         # more than have words of their own
+    assert bool((B.gemm(x, w) == 264).all())
+    ok(cu.cuCtxGetCurrent(C.byref(primary)))
+    ctx, scratch = C.c_void_p(), C.c_uint64()
+    ok(cu.cuCtxCreate_v2(C.byref(ctx), 0, 0))
+    ok(cu.cuMemAlloc_v2(C.byref(scratch), C.c_size_t(4096)))
+    for word, status in ((0, 0), (3, -6), (0, 0)):
+        ok(cu.cuMemsetD32_v2(scratch, word, C.c_size_t(1024)))
+        assert B.lib.specvla_gemm_status(C.c_void_p(scratch.value), None) == status
+    ok(cu.cuMemFree_v2(scratch))
+    ok(cu.cuCtxDestroy_v2(ctx))
+    ok(cu.cuCtxSetCurrent(primary))
+assert bool((B.gemm(x, w) == 264).all())
+"""
+
+
+def test_status_in_contexts_that_come_and_go():
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    done = subprocess.run([sys.executable, "-c", CONTEXTS], cwd=root, capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0, done.stderr[-2000:]
