@@ -1819,9 +1819,11 @@ int specvla_pack_weights(const void *W, int N, int K, void *packed, size_t packe
 struct DriverCalls {
   decltype(&cuCtxGetCurrent) current = nullptr;
   decltype(&cuCtxGetId) id = nullptr;
+  decltype(&cuPointerGetAttribute) attribute = nullptr;
   DriverCalls() {
     current = reinterpret_cast<decltype(current)>(find("cuCtxGetCurrent"));
     id = reinterpret_cast<decltype(id)>(find("cuCtxGetId"));
+    attribute = reinterpret_cast<decltype(attribute)>(find("cuPointerGetAttribute"));
   }
   static void *find(const char *name) {
     void *p = nullptr;
@@ -2017,16 +2019,25 @@ int specvla_gemm_static_status(void *stream) {
   return status_by_copy(reinterpret_cast<const void *>(base), static_cast<cudaStream_t>(stream));
 }
 
+// Whether a kernel launched now can read an int at p: aligned device memory of the current device and of the
+// current context. (Memory of a pool or of a mapped range has no context and is the device's.)
+static bool kernel_reads(const void *p) {
+  cudaPointerAttributes where = {};
+  int dev = -1;
+  if (reinterpret_cast<uintptr_t>(p) % alignof(int) != 0 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaPointerGetAttributes(&where, p) != cudaSuccess || where.type != cudaMemoryTypeDevice || where.device != dev)
+    return false;
+  const DriverCalls &cu = driver_calls();
+  CUcontext ctx = nullptr, owner = nullptr;
+  if (!cu.current || !cu.attribute || cu.current(&ctx) != CUDA_SUCCESS) return false;
+  if (cu.attribute(&owner, CU_POINTER_ATTRIBUTE_CONTEXT, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) owner = nullptr;
+  return !owner || owner == ctx;
+}
+
 int specvla_gemm_status(const void *scratch, void *stream) {
   if (!scratch) return SPECVLA_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the kernel reads memory of the device that is current; scratch that lies elsewhere is copied
-  cudaPointerAttributes where = {};
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&where, scratch) != cudaSuccess ||
-      where.type != cudaMemoryTypeDevice || where.device != dev)
-    return status_by_copy(scratch, st);
-  int *word = take_status_word();
+  int *word = kernel_reads(scratch) ? take_status_word() : nullptr;
   if (!word) return status_by_copy(scratch, st);
   cudaLaunchAttribute at;
   const cudaLaunchConfig_t cfg = launch_cfg(dim3(1), dim3(1), st, &at, true);

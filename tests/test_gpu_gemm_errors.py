@@ -141,6 +141,11 @@ for _ in range(20):                                         # more than have wor
     for word, status in ((0, 0), (3, -6), (0, 0)):
         ok(cu.cuMemsetD32_v2(scratch, word, C.c_size_t(1024)))
         assert B.lib.specvla_gemm_status(C.c_void_p(scratch.value), None) == status
+    ok(cu.cuMemsetD32_v2(scratch, 3, C.c_size_t(1024)))
+    ok(cu.cuCtxSynchronize())
+    ok(cu.cuCtxSetCurrent(primary))                         # memory of a context that is not the current one
+    assert B.lib.specvla_gemm_status(C.c_void_p(scratch.value), None) == -6
+    ok(cu.cuCtxSetCurrent(ctx))
     ok(cu.cuMemFree_v2(scratch))
     ok(cu.cuCtxDestroy_v2(ctx))
     ok(cu.cuCtxSetCurrent(primary))
@@ -152,3 +157,13 @@ def test_status_in_contexts_that_come_and_go():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     done = subprocess.run([sys.executable, "-c", CONTEXTS], cwd=root, capture_output=True, text=True, timeout=300)
     assert done.returncode == 0, done.stderr[-2000:]
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4])
+def test_status_of_a_word_at_any_address(offset):
+    """A word off a four-byte boundary is read as well."""
+    from paper_2507_22424_b200 import binding as B
+    buf = torch.zeros(64, dtype=torch.uint8, device="cuda")
+    for value, status in ((0, 0), (1, -6), (0, 0)):
+        buf[offset] = value
+        assert B.lib.specvla_gemm_status(C.c_void_p(buf.data_ptr() + offset), B._stream()) == status
