@@ -570,8 +570,9 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
       for (int sl = 0; sl < MAX_S; sl++) {
         // (Or what p held before would be kept in registers: 134 instead of 96 for the QKV mode of the wide
-        // Q8 block, which has 128. Where registers are not short it costs time: 128 bf16 rows +1.6 %.)
-        if (Q8) p[sl] = make_float4(0.f, 0.f, 0.f, 0.f);
+        // Q8 block, which has 128. Where registers are not short it costs time: 128 bf16 rows +1.6 %, 65 / 96 /
+        // 128 int8 rows 4.23 -> 4.35 / 4.69 -> 4.85 / 5.88 -> 5.97 ms.)
+        if (Q8 && q8_sets(TN) > 2) p[sl] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (sl < S) {
           // rank sl's copy of the same shared-memory address (mapped on the spot: an array of
           // eight mapped pointers would cost sixteen registers)
