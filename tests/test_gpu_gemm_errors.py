@@ -64,8 +64,8 @@ def test_a_wait_limit_covers_the_product_alone(T, N, K):
     assert (y.double() - ref).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
 
 
-def test_status_belongs_to_the_calling_thread():
-    """Products from several threads on streams of their own: each reads its own status and result."""
+def test_products_from_several_threads():
+    """Products from several threads on streams of their own: each succeeds with its own result."""
     from paper_2507_22424_b200.binding import gemm_prepacked, pack_weights
     g = torch.Generator().manual_seed(3)
     w = torch.randn(256, 264, generator=g).to(torch.bfloat16).cuda()
@@ -167,3 +167,78 @@ def test_status_of_a_word_at_any_address(offset):
     for value, status in ((0, 0), (1, -6), (0, 0)):
         buf[offset] = value
         assert B.lib.specvla_gemm_status(C.c_void_p(buf.data_ptr() + offset), B._stream()) == status
+
+
+def test_status_belongs_to_the_asking_thread():
+    """One product that timed out and one that did not, asked about at the same time by two threads."""
+    from paper_2507_22424_b200 import binding as B
+    T, N, K = 16, 256, 512
+    x, w, ref = _operands(T, N, K)
+    nb = B.lib.specvla_gemm_scratch_bytes(T, N, K)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    scratch = [torch.empty(nb + 1024, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    y = [torch.empty(T, N, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    at = [C.c_void_p((s.data_ptr() + 1023) // 1024 * 1024) for s in scratch]
+    on = [C.c_void_p(s.cuda_stream) for s in streams]
+    assert B.lib.specvla_gemm_fault_test(2_000_000, 1) == 0             # the first of the two products
+    for i in range(2):
+        assert B.lib.specvla_gemm(C.c_void_p(x.data_ptr()), C.c_void_p(w.data_ptr()), C.c_void_p(y[i].data_ptr()),
+                                  T, N, K, at[i], nb, on[i]) == 0
+    together, seen = threading.Barrier(2), [set(), set()]
+
+    def ask(i):
+        together.wait()
+        for _ in range(500):
+            seen[i].add(B.lib.specvla_gemm_status(at[i], on[i]))
+
+    threads = [threading.Thread(target=ask, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert seen == [{-6}, {0}], seen
+    assert (y[1].double() - ref).abs().max() < 1e-4 * 0.02 * (K ** 0.5) + 1e-6
+
+
+def test_more_calls_at_a_time_than_words():
+    """Seventy calls wait behind one kernel, each for its own word; twice, since the words come back."""
+    from paper_2507_22424_b200 import binding as B
+    n = 70
+    words = torch.zeros(n, 64, dtype=torch.int32, device="cuda")
+    words[::3] = 1
+    streams = [torch.cuda.Stream() for _ in range(n)]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        got = [None] * n
+        gate = torch.cuda.Event()
+        torch.cuda._sleep(200_000_000)                                  # about 0.1 s
+        gate.record()
+        for s in streams:
+            s.wait_event(gate)
+
+        def ask(i):
+            got[i] = B.lib.specvla_gemm_status(C.c_void_p(words[i].data_ptr()), C.c_void_p(streams[i].cuda_stream))
+
+        threads = [threading.Thread(target=ask, args=(i,)) for i in range(n)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert got == [-6 if i % 3 == 0 else 0 for i in range(n)], got
+
+
+def test_status_of_managed_memory():
+    """Memory that is not the device's own alone is copied."""
+    from paper_2507_22424_b200 import binding as B
+    torch.zeros(1, device="cuda")
+    cu = C.CDLL("libcuda.so.1")
+    scratch = C.c_uint64()
+    assert cu.cuMemAllocManaged(C.byref(scratch), C.c_size_t(4096), 1) == 0
+    try:
+        for value, status in ((0, 0), (1, -6), (0, 0)):
+            C.c_int.from_address(scratch.value).value = value
+            assert B.lib.specvla_gemm_status(C.c_void_p(scratch.value), B._stream()) == status
+            torch.cuda.synchronize()
+    finally:
+        assert cu.cuMemFree_v2(scratch) == 0

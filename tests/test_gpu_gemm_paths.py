@@ -39,10 +39,18 @@ def test_ring_sizes_of_long_tiles(T):
     _check(T, 20480, 1032, True)
 
 
-# several chunks: 88-row chunks of four stages with a shorter tail
+# several chunks with a tail box of the same width
 @pytest.mark.parametrize("T", [170, 176])
 def test_ring_sizes_of_several_chunks(T):
     _check(T, 4096, 2056, True)
+
+
+# a narrower tail box inside stages sized by the longer chunk: by the launch plan three chunks, unsplit, of 80
+# (tail 64) and 88 rows (72) in four stages, of 104 (96) and 120 rows (104) in three, and two of 80 (72) over K slices
+@pytest.mark.parametrize("T,N,K", [(220, 20480, 1032), (245, 20480, 1032), (300, 20480, 1032), (340, 20480, 1032),
+                                   (150, 4096, 2056)])
+def test_ring_with_a_narrower_tail(T, N, K):
+    _check(T, N, K, True)
 
 
 def test_operand_off_a_16_byte_boundary():

@@ -103,8 +103,9 @@ def test_withheld_key_tile(head_dim, tile):
     _exercise(Episodes(desc, [300 + 3 * i for i in range(14)], 41, 27), B.OPT_WITHHOLD_KEYS, tile)
 
 
-# first unit of either set of expanding warps, a later one, the first past the code ring, the last
-@pytest.mark.parametrize("unit", [0, 1, 6, 9, 15])
+# first unit of each of the three sets of expanding warps (64 rows at most), a later one of each, among them the
+# first past the code ring (8), the last
+@pytest.mark.parametrize("unit", [0, 1, 2, 6, 8, 9, 13, 15])
 @pytest.mark.parametrize("bits,rows", [(8, 9), (8, 60), (16, 9)])
 def test_withheld_weights(unit, bits, rows):
     """QKV of 128 K blocks over clusters of eight: sixteen units per CTA."""
