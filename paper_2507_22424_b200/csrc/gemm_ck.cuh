@@ -140,6 +140,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __shared__ __align__(16) float2 s_rope[ROPE_ROWS * ROPE_HALF];
   __shared__ float s_red[8][MAX_T];
   __shared__ int s_flag, s_fail;
+  __shared__ float s_sink;                 // values that no output takes (part 2)
   __shared__ float s_xv[4][2];             // EPI_TOPK: exchange between the two warps of a row group
   __shared__ int s_xi[4][2];
 
@@ -549,10 +550,10 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const int c4 = swiglu ? (et & 31) * 4 : (et & 63) * 4;    // first of the four columns within the tile
     const int n = swiglu ? tile * 128 + c4 : tile * BM + c4;
     const bool col_ok = n < ea.N;                             // N % 4 == 0: all four or none
-    // Peers' partial tiles are read only where something is stored that depends on them: the exit barrier
-    // below relies on it. (A scoring launch that returns no logits uses the columns of its id range alone.)
-    // The other threads read this CTA's own tile instead: a branch around the reads makes a verification
-    // call of 27 int8 rows 2 % slower (3.00 -> 3.06 ms), a prefill of 34 rows 0.5 %.
+    // Whether an output takes this thread's values. Where none does (columns past N, or outside the id range
+    // of a scoring launch that returns no logits) they go into a word of this CTA's shared memory instead: the
+    // exit barrier below relies on a store behind every read from a peer. (Reading such columns from this CTA's
+    // own tile cost sliced launches 0.3 to 0.5 %, a branch around the reads 27 int8 rows 2 %.)
     const bool used = col_ok && ((MODE != EPI_PLAIN && MODE != EPI_TOPK) || ea.out || (n + 3 >= ea.lo && n < ea.hi));
     const float *P_own = reinterpret_cast<const float *>(smem_raw + (base - smem_u32(smem_raw)));
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
@@ -576,7 +577,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (sl < S) {
           // rank sl's copy of the same shared-memory address (mapped on the spot: an array of
           // eight mapped pointers would cost sixteen registers)
-          const float *P = S == 1 ? P_own : cluster.map_shared_rank(const_cast<float *>(P_own), (unsigned)(used ? sl : rank));
+          const float *P = S == 1 ? P_own : cluster.map_shared_rank(const_cast<float *>(P_own), (unsigned)sl);
           p[sl] = *reinterpret_cast<const float4 *>(P + off);
         }
       }
@@ -770,6 +771,8 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           s2 = warp_sum(s2);
           if (lane == 0) s_red[warp - 2][t] = s2;
         }
+        if (!used)
+          asm volatile("st.shared.f32 [%0], %1;" ::"r"(smem_u32(&s_sink)), "f"(rot || swiglu ? v_[u].x + w_[u].x : v_[u].x) : "memory");
       }
     }
   }
@@ -777,7 +780,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // before leaving (nobody leaves while a peer may still be reading its shared memory), so that
   // the barrier's latency passes behind the rest of the epilogue. Relaxed: the barrier hands nothing over,
   // and a value that was read from a peer has arrived, because a store that depends on it has been issued
-  // (`used` above: no such read is without one). A releasing arrival makes every warp wait until
+  // (`used` above: no read is without one). A releasing arrival makes every warp wait until
   // the tile's stores to global memory are through, before a barrier that the peers wait for: verification of
   // 1 / 27 / 60 rows 2.73 / 2.99 / 3.54 ms with it here and in the few-row attention, 2.63 / 2.92 / 3.50 without.
   if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");

@@ -1,5 +1,5 @@
 """Sliced launches whose last tile is partly past the matrix, or whose tiles are partly outside the scored id
-range: a thread takes its peers' partial sums only where it stores something that depends on them."""
+range: threads whose values no output takes read their peers' partial sums like the others."""
 import pytest
 import torch
 
