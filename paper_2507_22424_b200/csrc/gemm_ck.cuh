@@ -59,7 +59,7 @@ __device__ __forceinline__ void cluster_sync_all() {
 // in shared memory, whose three 32 KB buffers, block barriers and proxy fences bounded the kernel: a
 // verification call of 27 rows took 3.19 ms instead of 4.45, of 8 rows 3.04 instead of 4.23, of 97 rows
 // 5.63 instead of 6.16. A unit then took a CTA 0.45 us at every width up to 32 rows, the two sets of warps
-// of the epilogue taking turns; a third set (below) makes that 0.43 (27 rows 3.22 -> 3.11 ms, one row
+// of the epilogue taking turns; a third set (below) makes that 0.43 (27 rows 3.22 -> 3.10 ms, one row
 // 3.01 -> 2.89, 60 rows 3.75 -> 3.68). A fourth set, six expanded buffers instead of four, and copies of
 // a sixteenth of the codes change nothing more; with the conversion left out a unit takes 0.35 us, without the
 // stores to TMEM 0.30: what bounds it is instructions, two logical operations and a subtraction per two
@@ -97,7 +97,7 @@ __device__ __forceinline__ uint32_t codes_to_bf16x2(uint32_t w) {
 // The long bf16 instantiation sizes its stages by the rows of its chunks (a tail has no more), and has four
 // of them up to 88 rows, three above: the most that fit beside the kernel's static shared memory. Three
 // stages of 64 KB, whatever the rows, did not cover the latency of the weights at 65 to 88 rows, where the
-// MMAs take less than they do: a verification step of 70 rows 4.16 -> 4.01 ms. (Rings of their own for
+// MMAs take less than they do: a verification step of 70 rows 4.35 -> 4.13 ms. (Rings of their own for
 // weights and X, four to six slots of one and two to four of the other, cost a second commit and a second
 // wait per K block: 96 rows -1 %, a prefill of 290 rows +3.5 %.)
 constexpr int LONG_STAGES = 4, LONG_RING = 216 * 1024;
@@ -917,8 +917,9 @@ inline int slices_for(int units, int KB, const ClusterFit &fit) {
 // clocks: waves x (fixed part of a CTA + its K blocks x clocks per K block), where a K block of tn
 // rows costs 512 + 6 tn clocks (what its 64 KB + 768 tn bytes of shared-memory traffic take at
 // 128 bytes per clock; the MMAs themselves need 8 tn). Fitted on a kernel that issued its MMAs under a
-// one-lane branch; the current one takes about 800 clocks at 80 rows, where this counts 992. int8
-// launches, whose shared-memory traffic is another, use the same estimate.
+// one-lane branch and had three ring stages at every size; the current one, with four up to 88 rows, takes
+// 655 clocks at 80 rows, where this counts 992. It does not know the two rings apart, and int8 launches,
+// whose shared-memory traffic is another, use the same estimate.
 struct RowPlan {
   int chunks, chunk_rows, tn_chunk, tn_tail, S;
 };
